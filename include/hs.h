@@ -523,7 +523,10 @@ hs_status hs_profile_read(hs_ctx ctx, double* phase_ms, double* phase_flops, int
 /* C[M, N] = A[M, K] B[N, K]^T for row-major FP64 device matrices with leading
  * dimensions lda >= K, ldb >= K, ldc >= N: the dense GEMM that the Z2 block
  * contraction performs inside one parity block. HS_PREC_F64 runs the FP64
- * kernel; the TF32/BF16 modes split A and B into hi/lo parts (padded copies in
+ * kernel, or, where the product is large enough to pay for it, sums of exact
+ * digit products on the tensor cores whose error is not larger than that of an
+ * FP64 chain (never on a stream under capture; the operands' digits are kept in
+ * the context workspace, at most 1 GiB); the TF32/BF16 modes split A and B into hi/lo parts (padded copies in
  * the context workspace) and run the tcgen05 tensor-core kernel with FP32
  * accumulation, writing FP64. Asynchronous; a timed-out device wait is
  * reported by the next hs_sync as HS_ERR_TIMEOUT. */

@@ -2,6 +2,7 @@
 // arXiv 2410.11596 (Sec. II.A, Fig. 1(d)) in the Hermitian Z2 basis
 // (Sec. II.B).
 #include <algorithm>
+#include <climits>
 #include <utility>
 
 #include "hs_ctx.cuh"
@@ -61,10 +62,141 @@ hs_status gemm(hs_ctx ctx, hs_gemm_backend be, const GemmGroup& g, const double*
     }
     return HS_OK;
   }
+  return gemm_f64(ctx, g, A, B, C);
+}
+
+hs_status gemm_dfma(hs_ctx ctx, const GemmGroup& g, const double* A, const double* B, double* C, double alpha,
+                    bool accumulate) {
   HS_TRY(ctx->splitk.ensure(kSplitKElems * sizeof(double)));
-  HS_CUDA(launch_gemm_f64(g, A, B, C, 1.0, ctx->stream, ctx->splitk.d(), kSplitKElems));
+  HS_CUDA(launch_gemm_f64(g, A, B, C, alpha, ctx->stream, ctx->splitk.d(), kSplitKElems, accumulate));
   if (g.n > 0) ctx->launches += 1;
   return HS_OK;
+}
+
+namespace {
+// The digit slices' workspace per context, at most. Larger products run in
+// panels of rows whose slices fill half of it (the other operand's in the rest).
+constexpr size_t kSliceBytes = size_t(1) << 30;
+
+// A stream under capture gets the FP64 kernel: it needs no workspace that a
+// later call could outgrow while the graph still points to it.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
+SlMat row_panel(const SlMat& m, int r0, int rows) {
+  SlMat v = m;
+  v.p[0] += (long long)r0 * m.ld;
+  if (m.nseg > 1) v.p[1] += (long long)r0 * m.ld;
+  v.rows = rows;
+  return v;
+}
+
+int operand(SlMat* mats, int* n, const SlMat& m) {
+  for (int i = 0; i < *n; ++i) {
+    const SlMat& o = mats[i];
+    if (o.is_b == m.is_b && o.p[0] == m.p[0] && o.nseg == m.nseg && o.kseg == m.kseg && o.rows == m.rows && o.ld == m.ld &&
+        o.neg[0] == m.neg[0] && (m.nseg < 2 || (o.p[1] == m.p[1] && o.neg[1] == m.neg[1])))
+      return i;
+  }
+  mats[*n] = m;
+  return (*n)++;
+}
+
+// The products on the tensor cores by digit slices when that is the faster
+// way; *done = false leaves them to the FP64 kernel.
+hs_status gemm_sliced(hs_ctx ctx, const SlMat* mats, int nm, const SlProblem* probs, int np,
+                      bool accumulate, bool* done) {
+  *done = false;
+  if (np < 1 || ctx->no_slices || !slices_pay(probs, mats, np) || capturing(ctx->stream)) return HS_OK;
+  size_t all = 0;
+  for (int i = 0; i < nm; ++i) all += slices_bytes(mats[i].rows, mats[i].kseg * mats[i].nseg, mats[i].is_b);
+  if (ctx->sl_ws.ensure(all < kSliceBytes ? all : kSliceBytes) != HS_OK) return HS_OK;  // no memory left
+  int* err = static_cast<int*>(ctx->tc_err.p);
+  if (all <= ctx->sl_ws.bytes) {
+    HS_CUDA(launch_gemm_slices(mats, nm, probs, np, accumulate, ctx->sl_ws.p, ctx->sl_ws.bytes, err,
+                               ctx->stream));
+    ctx->launches += 2;
+    *done = true;
+    return HS_OK;
+  }
+  const size_t half = ctx->sl_ws.bytes / 2;
+  for (int i = 0; i < np; ++i) {
+    const SlMat &a = mats[probs[i].a], &b = mats[probs[i].b];
+    auto panel = [&](const SlMat& m) {
+      const int block = slices_block(m.is_b);
+      const long long r = (long long)(half / slices_bytes(block, m.kseg * m.nseg, m.is_b)) * block;
+      return (int)(r < m.rows ? r : m.rows);
+    };
+    const int ra = panel(a), rb = panel(b);
+    if (ra < 1 || rb < 1) return fail(HS_ERR_SHAPE, "contraction of %d too long for the slices", a.kseg * a.nseg);
+    for (int n0 = 0; n0 < b.rows; n0 += rb)
+      for (int m0 = 0; m0 < a.rows; m0 += ra) {
+        const SlMat part[2] = {row_panel(a, m0, std::min(ra, a.rows - m0)), row_panel(b, n0, std::min(rb, b.rows - n0))};
+        const SlProblem pr = {0, 1, probs[i].c + (long long)m0 * probs[i].ldc + n0, probs[i].ldc};
+        HS_CUDA(launch_gemm_slices(part, 2, &pr, 1, accumulate, ctx->sl_ws.p, ctx->sl_ws.bytes, err,
+                                   ctx->stream));
+        ctx->launches += 2;
+      }
+  }
+  *done = true;
+  return HS_OK;
+}
+}  // namespace
+
+namespace {
+hs_status gemm_try_sliced(hs_ctx ctx, const GemmGroup& g, const double* A, const double* B, double* C,
+                          bool accumulate, bool* done) {
+  *done = false;
+  SlMat mats[2 * kMaxProblems];
+  SlProblem probs[kMaxProblems];
+  int nm = 0, np = 0;
+  for (int i = 0; i < g.n; ++i) {
+    const GemmProblem& p = g.p[i];
+    if (p.M <= 0 || p.N <= 0) continue;
+    if (p.K <= 0) return HS_OK;
+    SlProblem& q = probs[np++];
+    q.a = operand(mats, &nm, SlMat{{A + p.a_off, nullptr}, {false, false}, 1, p.K, p.M, p.lda, false});
+    q.b = operand(mats, &nm, SlMat{{B + p.b_off, nullptr}, {false, false}, 1, p.K, p.N, p.ldb, true});
+    q.c = C + p.c_off;
+    q.ldc = p.ldc;
+  }
+  return gemm_sliced(ctx, mats, nm, probs, np, accumulate, done);
+}
+}  // namespace
+
+hs_status gemm_f64(hs_ctx ctx, const GemmGroup& g, const double* A, const double* B, double* C, bool accumulate) {
+  bool done = false;
+  HS_TRY(gemm_try_sliced(ctx, g, A, B, C, accumulate, &done));
+  return done ? HS_OK : gemm_dfma(ctx, g, A, B, C, 1.0, accumulate);
+}
+
+hs_status zgemm_f64(hs_ctx ctx, const GemmGroup& g, const double* Ar, const double* Ai, const double* Br,
+                    const double* Bi, double* Cr, double* Ci, bool conj_b) {
+  if (g.n == 1 && g.p[0].M > 0 && g.p[0].N > 0 && g.p[0].K > 0 && g.p[0].K <= INT_MAX / 2) {
+    // Re C = [Re A | Im A] [Re B | -Im B]^T, Im C = [Re A | Im A] [Im B | Re B]^T
+    // (Im B negated for conj(B)): one product with the contraction doubled
+    const GemmProblem& p = g.p[0];
+    const SlMat mats[3] = {
+        SlMat{{Ar + p.a_off, Ai + p.a_off}, {false, false}, 2, p.K, p.M, p.lda, false},
+        SlMat{{Br + p.b_off, Bi + p.b_off}, {false, !conj_b}, 2, p.K, p.N, p.ldb, true},
+        SlMat{{Bi + p.b_off, Br + p.b_off}, {conj_b, false}, 2, p.K, p.N, p.ldb, true},
+    };
+    const SlProblem probs[2] = {{0, 1, Cr + p.c_off, p.ldc}, {0, 2, Ci + p.c_off, p.ldc}};
+    bool done = false;
+    HS_TRY(gemm_sliced(ctx, mats, 3, probs, 2, false, &done));
+    if (done) return HS_OK;
+  }
+  const double sb = conj_b ? -1.0 : 1.0;
+  HS_TRY(gemm_dfma(ctx, g, Ar, Br, Cr, 1.0, false));
+  HS_TRY(gemm_dfma(ctx, g, Ai, Bi, Cr, -sb, true));
+  HS_TRY(gemm_dfma(ctx, g, Ar, Bi, Ci, sb, false));
+  return gemm_dfma(ctx, g, Ai, Br, Ci, 1.0, true);
 }
 
 // make_perm_plan through the context's cache, keyed by the two layouts and
@@ -522,8 +654,8 @@ hs_status finish_projector(hs_ctx ctx, int n0, int n1, SelectOut* dsel, Sect c, 
     GemmGroup gc = group([&](int p) {
       return GemmProblem{k[p], k[p], n[p], n[p], n[p], k[p], ptoff[p], ptoff[p], goff[p]};
     });
-    HS_CUDA(launch_gemm_f64(gw, PT, C0, W, 1.0, s, ctx->splitk.d(), kSplitKElems));
-    HS_CUDA(launch_gemm_f64(gc, W, PT, env->C, 1.0, s, ctx->splitk.d(), kSplitKElems));
+    HS_TRY(gemm_f64(ctx, gw, PT, C0, W));
+    HS_TRY(gemm_f64(ctx, gc, W, PT, env->C));
     *flops += gemm_flops(gw) + gemm_flops(gc);
     ctx->phase_flops[HS_PHASE_GEMM] += gemm_flops(gw) + gemm_flops(gc);
   } else {
@@ -685,12 +817,12 @@ hs_status orthonormalise_rows(hs_ctx ctx, hs_precision prec, double* const X[2],
   if (stacked) {
     GemmGroup gg{2, {GemmProblem{m[0], m[0], n[0], n[0], n[0], m[0], 0, 0, 0},
                      GemmProblem{m[1], m[1], n[1], n[1], n[1], m[1], mn0, mn0, G[1] - G[0]}}};
-    HS_TRY(gemm(ctx, HS_GEMM_OWN, gg, X[0], X[0], G[0]));
+    HS_TRY(gemm_dfma(ctx, gg, X[0], X[0], G[0]));
   } else {
     for (int b = 0; b < 2; ++b)
       if (m[b] > 0)
-        HS_TRY(gemm(ctx, HS_GEMM_OWN, GemmGroup{1, {GemmProblem{m[b], m[b], n[b], n[b], n[b], m[b], 0, 0, 0}}},
-                    X[b], X[b], G[b]));
+        HS_TRY(gemm_dfma(ctx, GemmGroup{1, {GemmProblem{m[b], m[b], n[b], n[b], n[b], m[b], 0, 0, 0}}}, X[b], X[b],
+                         G[b]));
   }
   if (mm <= max_chol()) {
     HS_CUDA(launch_chol_inv(G[0], m[0], Li[0], G[1], m[1], Li[1], bad, ctx->stream));
@@ -726,15 +858,15 @@ hs_status orthonormalise_rows(hs_ctx ctx, hs_precision prec, double* const X[2],
     HS_TRY(permute(ctx, zd(m[0], m[1], n[0], n[1]), zd(n[0], n[1], m[0], m[1]), {1, 0}, X[0], Xc[0]));
     GemmGroup gl{2, {GemmProblem{m[0], n[0], m[0], m[0], m[0], n[0], 0, 0, 0},
                      GemmProblem{m[1], n[1], m[1], m[1], m[1], n[1], Li[1] - Li[0], mn0, mn0}}};
-    HS_TRY(gemm(ctx, HS_GEMM_OWN, gl, Li[0], Xc[0], X[0]));
+    HS_TRY(gemm_dfma(ctx, gl, Li[0], Xc[0], X[0]));
     HS_TRY(lowdin_rows_pair(ctx, prec, X[0], m, n, Xc[0], 1));
     return HS_OK;
   }
   for (int b = 0; b < 2; ++b)
     if (m[b] > 0) {
       HS_TRY(permute(ctx, dense2(m[b], n[b]), dense2(n[b], m[b]), {1, 0}, X[b], Xc[b]));
-      HS_TRY(gemm(ctx, HS_GEMM_OWN, GemmGroup{1, {GemmProblem{m[b], n[b], m[b], m[b], m[b], n[b], 0, 0, 0}}},
-                  Li[b], Xc[b], X[b]));
+      HS_TRY(gemm_dfma(ctx, GemmGroup{1, {GemmProblem{m[b], n[b], m[b], m[b], m[b], n[b], 0, 0, 0}}}, Li[b], Xc[b],
+                       X[b]));
       HS_TRY(lowdin_rows(ctx, prec, X[b], m[b], n[b], Xc[b], 1));
     }
   return HS_OK;
@@ -1509,7 +1641,7 @@ hs_status hs_destroy(hs_ctx ctx) {
   ctx->ps_hi.release();
   ctx->ps_lo.release();
   DBuf* more[] = {&ctx->c32,  &ctx->w32,   &ctx->pcol,         &ctx->pt2,   &ctx->gram,
-                  &ctx->wproj, &ctx->solver32_dev, &ctx->splitk, &ctx->ws_pt, &ctx->sth,
+                  &ctx->wproj, &ctx->solver32_dev, &ctx->splitk, &ctx->sl_ws, &ctx->ws_pt, &ctx->sth,
                   &ctx->sx_hi, &ctx->sx_lo, &ctx->sy_hi, &ctx->sy_lo, &ctx->schol};
   for (Stacked* t : {&ctx->sx, &ctx->sz, &ctx->sxc, &ctx->szc, &ctx->sxr, &ctx->szr, &ctx->sbm, &ctx->sbw, &ctx->sres})
     t->release();
@@ -1742,6 +1874,10 @@ hs_status hs_ctmrg_move(hs_ctx ctx, const hs_z2_tensor* a, hs_env* env, int chi,
     return fail(HS_ERR_SHAPE, "tensor and environment disagree on D or basis");
   if (chi < 1 || chi > env->chi_max) return fail(HS_ERR_SHAPE, "chi %d outside [1, %d]", chi, env->chi_max);
   if (env->dtype != a->dtype) return fail(HS_ERR_DTYPE, "tensor and environment disagree on dtype");
+  // The iterative projectors stop at a residual of 1e-6, so their environments
+  // depend on the products' last bits at the level of the energies' gates
+  // (1e-8): they keep the FP64 kernel's summation order
+  NoSlices keep(ctx, env->eig_mode != HS_EIG_F64);
   if (env->dtype == HS_C128)
     return env->basis == HS_BASIS_DENSE ? zdense_move(ctx, a, env, chi, info) : graded_move(ctx, a, env, chi, info);
   cudaStream_t s = ctx->stream;
@@ -2127,7 +2263,9 @@ hs_status hs_gemm(hs_ctx ctx, hs_precision precision, int M, int N, int K, const
     GemmGroup g{};
     g.n = 1;
     g.p[0] = GemmProblem{M, N, K, lda, ldb, ldc, 0, 0, 0};
-    HS_CUDA(launch_gemm_f64(g, A, B, C, 1.0, ctx->stream));
+    bool done = false;
+    HS_TRY(gemm_try_sliced(ctx, g, A, B, C, false, &done));
+    if (!done) HS_CUDA(launch_gemm_f64(g, A, B, C, 1.0, ctx->stream));
     return HS_OK;
   }
   if (precision != HS_PREC_TF32X3 && precision != HS_PREC_TF32 && precision != HS_PREC_BF16X3)

@@ -296,4 +296,52 @@ HS_HD bool f32_widen_fast(uint32_t f, unsigned long long& out) {
   return true;
 }
 
+// ---- FP64 operands as slices of 8-bit digits (k_gemm_sl.cu) -------------------
+//
+// A row whose largest biased exponent field is emax is written as
+//   x = 2^(emax - 1022 - 55) X,  |X| < 2^55 an integer (rounded to nearest),
+//   X = sum_{i=1..7} d_i 256^(7 - i),  d_i in [-128, 127] (d_1 up to 128),
+// so that slice i holds the integers d_i, exact in BF16.
+
+// X of x for a row whose largest exponent field is emax (x finite, emax >= 1).
+HS_HD long long slice_fixed(double x, int emax) {
+  const unsigned long long b = f64_bits(x);
+  int E = (int)((b >> 52) & 0x7FF);
+  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+  if (E)
+    m |= 1ull << 52;
+  else
+    E = 1;  // subnormal
+  const int d = emax - E;  // >= 0
+  unsigned long long v;
+  if (d <= 2) {
+    v = m << (2 - d);
+  } else {
+    const int r = d - 2;
+    v = r <= 54 ? (m + (1ull << (r - 1))) >> r : 0ull;
+  }
+  return (b >> 63) ? -(long long)v : (long long)v;
+}
+
+// Y = X + sum of 128 at the six lower digits: d_i = byte (7 - i) of Y minus 128
+// for i = 2..7, d_1 = Y >> 48 (arithmetic).
+HS_HD long long slice_bias(long long X) { return X + 0x808080808080ll; }
+
+// Digit d_i (i = 1..7) of the biased value.
+HS_HD int slice_digit(long long Y, int i) {
+  return i == 1 ? (int)(Y >> 48) : (int)((unsigned long long)Y >> (8 * (7 - i)) & 0xFF) - 128;
+}
+
+// Bit pattern of the double J 2^s, |J| < 2^63, rounded to nearest even; 0 for
+// J = 0. The caller keeps the result in the normal range.
+HS_HD unsigned long long fixed_to_f64(long long J, int s) {
+  const unsigned long long sign = (unsigned long long)J & (1ull << 63);
+  const unsigned long long mag = J < 0 ? 0ull - (unsigned long long)J : (unsigned long long)J;
+  const int lz = clz64(mag | 1) - 1;         // top bit to 62
+  const unsigned long long n = mag << lz;
+  const unsigned long long q = (n + 0x1FF + ((n >> 10) & 1)) >> 10;  // 53 bits, or 2^53
+  // the implicit bit of q (or its carry into 2^53) adds to the exponent field
+  return mag == 0 ? 0ull : sign | (((unsigned long long)(62 - lz + s + 1022) << 52) + q);
+}
+
 }  // namespace hs

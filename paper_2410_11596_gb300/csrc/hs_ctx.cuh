@@ -176,8 +176,9 @@ struct hs_ctx_s {
   gesvdjInfo_t gesvdj = nullptr;
   std::vector<char> d4_work_host;
   long long d4_svd_fallbacks = 0;  // blocks that took the Jacobi SVD
-  // split-K partial sums of the FP64 GEMM
-  hs::DBuf splitk;
+  // split-K partial sums of the FP64 GEMM, digit slices of its operands
+  hs::DBuf splitk, sl_ws;
+  bool no_slices = false;  // this call's FP64 products all take the FP64 kernel (NoSlices)
   // subspace eigensolver: warm start (previous kept rows, per block) and
   // per-block iteration buffers
   const void* ws_env = nullptr;
@@ -241,11 +242,26 @@ struct hs_ctx_s {
 namespace hs {
 
 hs_status check_ctx(hs_ctx ctx);
+// While it lives (one call), the context's FP64 products take the FP64 kernel if `off`.
+struct NoSlices {
+  hs_ctx c;
+  NoSlices(hs_ctx ctx, bool off) : c(ctx) { c->no_slices = off; }
+  ~NoSlices() { c->no_slices = false; }
+};
 Sect q_sect(int D, hs_basis b);
 Z2Mat mat(Fused r, Fused c, int pad = 1);
 // C = A B^T on the chosen backend.
 hs_status gemm(hs_ctx ctx, hs_gemm_backend be, const GemmGroup& g, const double* A, const double* B,
                double* C);
+// C = A B^T (+ C) in FP64: by digit slices on the tensor cores where they
+// win (slices_pay), else on the FP64 kernel; gemm_dfma takes the FP64 kernel always.
+hs_status gemm_f64(hs_ctx ctx, const GemmGroup& g, const double* A, const double* B, double* C,
+                   bool accumulate = false);
+hs_status gemm_dfma(hs_ctx ctx, const GemmGroup& g, const double* A, const double* B, double* C, double alpha = 1.0,
+                    bool accumulate = false);
+// Complex C = A B^T (or A conj(B)^T) of planar FP64 parts.
+hs_status zgemm_f64(hs_ctx ctx, const GemmGroup& g, const double* Ar, const double* Ai, const double* Br,
+                    const double* Bi, double* Cr, double* Ci, bool conj_b);
 // make_perm_plan through the context's cache (perm: kMaxLegs entries).
 const PermPlan& cached_plan(hs_ctx ctx, const Z2Mat& in, const Z2Mat& out, const int* perm);
 // The open double layers of the two-site network and their adjoint (dA =, not +=).

@@ -187,11 +187,7 @@ hs_status permute_p(hs_ctx ctx, const Z2Mat& in, const Z2Mat& out, const int* p,
 
 hs_status gemm_acc(hs_ctx ctx, const Z2Mat& Am, const double* A, const Z2Mat& Bm, const double* B, const Z2Mat& Cm,
                    double* C, bool acc) {
-  HS_TRY(ctx->splitk.ensure(kSplitKElems * sizeof(double)));
-  const GemmGroup g = make_z2_gemm(Am, Bm, Cm);
-  HS_CUDA(launch_gemm_f64(g, A, B, C, 1.0, ctx->stream, ctx->splitk.d(), kSplitKElems, acc));
-  if (g.n > 0) ctx->launches += 1;
-  return HS_OK;
+  return gemm_f64(ctx, make_z2_gemm(Am, Bm, Cm), A, B, C, acc);
 }
 
 // C = A B^T (layouts Am [R|K], Bm [N|K], Cm [R|N]); reverse: dA += dC B, dB += dC^T A

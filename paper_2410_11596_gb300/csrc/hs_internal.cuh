@@ -388,6 +388,31 @@ cudaError_t launch_gemm_f64(const GemmGroup& g, const double* A, const double* B
                             double alpha, cudaStream_t s, double* part = nullptr, long long part_elems = 0,
                             bool accumulate = false);
 
+// FP64 GEMM by digit slices on the tensor cores (k_gemm_sl.cu). One operand: a
+// rows x (nseg kseg) matrix whose columns come from one or two row-major
+// sources of the same row stride, each negated where neg is set (two sources:
+// the real and imaginary parts of a complex operand).
+struct SlMat {
+  const double* p[2];
+  bool neg[2];
+  int nseg, kseg, rows;
+  long long ld;
+  bool is_b;  // an N-side operand (its digit planes are laid out in other row blocks)
+};
+// C[rows of mats[a], rows of mats[b]] = A B^T (+ C).
+struct SlProblem {
+  int a, b;
+  double* c;
+  int ldc;
+};
+// Workspace bytes of one operand (rows in whole blocks when it is a panel); whether the slices beat the FP64 kernel.
+size_t slices_bytes(int rows, int K, bool is_b);
+int slices_block(bool is_b);  // rows per block of the planes
+bool slices_pay(const SlProblem* probs, const SlMat* mats, int n);
+// Up to 8 operands and 4 problems per call (K <= 65536); err as for launch_gemm_tc.
+cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob,
+                               bool accumulate, void* ws, size_t ws_bytes, int* err, cudaStream_t s);
+
 // A[p,u,l,d,r] (real) -> a~ blocks in FSO [(u,l)|(d,r)]; hermitian selects the
 // rotation by U^T on every leg, otherwise the plain combined basis.
 cudaError_t launch_double_layer_blocks(const double* A, int d, int D, bool hermitian, double* out,

@@ -342,18 +342,9 @@ ZBuf zbuf(hs_ctx ctx, int i, long long n) {
   return {ctx->zr[2 * i].d(), ctx->zr[2 * i + 1].d()};
 }
 
-// complex C = A B^T (or A conj(B)^T) from planar parts: four FP64 GEMMs, two accumulating
+// complex C = A B^T (or A conj(B)^T) from planar parts
 hs_status zgemm(hs_ctx ctx, const GemmGroup& g, ZBuf A, ZBuf B, ZBuf C, bool conj_b = false) {
-  cudaStream_t s = ctx->stream;
-  HS_TRY(ctx->splitk.ensure(kSplitKElems * sizeof(double)));
-  double* part = ctx->splitk.d();
-  const double sb = conj_b ? -1.0 : 1.0;
-  HS_CUDA(launch_gemm_f64(g, A.re, B.re, C.re, 1.0, s, part, kSplitKElems, false));
-  HS_CUDA(launch_gemm_f64(g, A.im, B.im, C.re, -sb, s, part, kSplitKElems, true));
-  HS_CUDA(launch_gemm_f64(g, A.re, B.im, C.im, sb, s, part, kSplitKElems, false));
-  HS_CUDA(launch_gemm_f64(g, A.im, B.re, C.im, 1.0, s, part, kSplitKElems, true));
-  ctx->launches += 4;
-  return HS_OK;
+  return zgemm_f64(ctx, g, A.re, A.im, B.re, B.im, C.re, C.im, conj_b);
 }
 
 // dA of a complex A from the cotangents g1, g2 of the two open double layers

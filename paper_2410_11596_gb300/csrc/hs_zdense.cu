@@ -124,21 +124,13 @@ Z2Mat dn(std::initializer_list<long long> dims) {
   return mat(r, c);
 }
 
-// C = A B^T (or A conj(B)^T) for M x K and N x K planar complex operands: four FP64 GEMMs
+// C = A B^T (or A conj(B)^T) for M x K and N x K planar complex operands
 hs_status zmul(hs_ctx ctx, long long M, long long N, long long K, ZB A, ZB B, ZB C, bool conj_b, double* flops) {
-  cudaStream_t s = ctx->stream;
   GemmGroup g{};
   g.n = 1;
   g.p[0] = GemmProblem{(int)M, (int)N, (int)K, (int)K, (int)K, (int)N, 0, 0, 0};
-  HS_TRY(ctx->splitk.ensure(kSplitKElems * sizeof(double)));
-  double* part = ctx->splitk.d();
-  const double sb = conj_b ? -1.0 : 1.0;
   PhaseScope ps(ctx, HS_PHASE_GEMM);
-  HS_CUDA(launch_gemm_f64(g, A.re, B.re, C.re, 1.0, s, part, kSplitKElems, false));
-  HS_CUDA(launch_gemm_f64(g, A.im, B.im, C.re, -sb, s, part, kSplitKElems, true));
-  HS_CUDA(launch_gemm_f64(g, A.re, B.im, C.im, sb, s, part, kSplitKElems, false));
-  HS_CUDA(launch_gemm_f64(g, A.im, B.re, C.im, 1.0, s, part, kSplitKElems, true));
-  ctx->launches += 4;
+  HS_TRY(zgemm_f64(ctx, g, A.re, A.im, B.re, B.im, C.re, C.im, conj_b));
   const double f = 8.0 * M * (double)N * K;
   *flops += f;
   ctx->phase_flops[HS_PHASE_GEMM] += f;

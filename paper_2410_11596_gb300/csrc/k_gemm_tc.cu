@@ -41,6 +41,7 @@
 
 #include "hs_bits.cuh"
 #include "hs_internal.cuh"
+#include "hs_tc.cuh"
 
 namespace hs {
 
@@ -51,7 +52,6 @@ constexpr int kEpiWarps = 8;              // two per TMEM lane quarter, each on 
 constexpr int NT = 32 * (2 + kEpiWarps);  // TMA warp, MMA warp, epilogue warps
 constexpr int ROW_BYTES = 128;
 constexpr int TILE_BYTES = BM * ROW_BYTES;  // BN == BM
-constexpr long long WAIT_LIMIT = 20000000;  // try_wait rounds before giving up (seconds)
 
 constexpr int kMaxPairs = 4;  // operand pairs of one launch (the four graded sub-products)
 template <int NM>
@@ -89,61 +89,6 @@ __device__ __forceinline__ int ps_co(const PsDesc& D, int tr, int tc, int k) {
   return tr ? D.co[1][tc][k] : D.co[0][tc][k];
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait (limit try_wait rounds); on timeout records the code and
-// raises the abort flag.
-__device__ __forceinline__ bool mbar_wait_n(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                            int* err, int code, long long limit) {
-  for (long long i = 0; i < limit; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-  }
-  *abort_flag = 1;
-  atomicExch(err, code);
-  return false;
-}
-
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          int* err, int code) {
-  return mbar_wait_n(bar, parity, abort_flag, err, code, WAIT_LIMIT);
-}
-
-// Drain wait after an abort: bounded, never raises anything.
-__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
-  for (long long i = 0; i < WAIT_LIMIT; ++i)
-    if (mbar_try(bar, parity)) return;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
-                                            uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-      "[%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
-      : "memory");
-}
-
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row core
 // groups 1024 bytes apart (rows are 128 bytes), descriptor version 1.
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
@@ -177,18 +122,6 @@ __device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uin
   }
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -200,8 +133,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
-
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 template <int NPASS, int EB>
 struct Cfg {
@@ -229,10 +160,6 @@ __device__ __forceinline__ TileRef tile_of(const Group& g, int t) {
   while (pi + 1 < g.n && t >= g.p[pi + 1].tile_start) ++pi;
   t -= g.p[pi].tile_start;
   return {pi, (t / g.p[pi].tiles_n) * BM, (t % g.p[pi].tiles_n) * BN};
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 template <int NPASS, int EB, int NM, bool PS>
@@ -603,20 +530,6 @@ __global__ void __launch_bounds__(NT, 1) gemm_tc_kernel(const __grid_constant__ 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(K::TMEM_COLS)
                  : "memory");
   }
-}
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  });
-  return fn;
 }
 
 // 2-D map over a row-major [rows, Kp] operand, box = 128 rows x 128 bytes.
