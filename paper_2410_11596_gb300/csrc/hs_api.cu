@@ -2265,7 +2265,10 @@ hs_status hs_gemm(hs_ctx ctx, hs_precision precision, int M, int N, int K, const
     g.p[0] = GemmProblem{M, N, K, lda, ldb, ldc, 0, 0, 0};
     bool done = false;
     HS_TRY(gemm_try_sliced(ctx, g, A, B, C, false, &done));
-    if (!done) HS_CUDA(launch_gemm_f64(g, A, B, C, 1.0, ctx->stream));
+    if (done) return HS_OK;
+    // (split K needs the context's workspace, which a capture may not allocate)
+    if (!capturing(ctx->stream)) return gemm_dfma(ctx, g, A, B, C);
+    HS_CUDA(launch_gemm_f64(g, A, B, C, 1.0, ctx->stream));
     return HS_OK;
   }
   if (precision != HS_PREC_TF32X3 && precision != HS_PREC_TF32 && precision != HS_PREC_BF16X3)

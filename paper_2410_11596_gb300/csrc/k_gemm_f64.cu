@@ -1,7 +1,9 @@
 // Grouped FP64 GEMM (DFMA) for the block contractions in FP64 mode:
 // C[m, n] = alpha * sum_k A[m, k] B[n, k] (+ C[m, n] when accumulating), both
 // operands K-major (row-major M x K and N x K). One CTA per 64 x 64 output
-// tile of any problem of the group.
+// tile of any problem of the group, or per 16 x 16 tile where that spreads the
+// work better (launch_gemm_f64). Every entry is the same chain of FMAs over k
+// in both.
 #include "hs_internal.cuh"
 
 namespace hs {
@@ -99,6 +101,62 @@ __global__ void __launch_bounds__(NT) gemm_f64_nt_kernel(GemmGroup g, const doub
   }
 }
 
+// The same products on 16 x 16 tiles, one entry per thread. The FP64 pipe does 1.7
+// FMAs per clock and SM, so a 64 x 64 x 64 tile takes 75 us wherever it runs and
+// padding costs as much as work; loads are cheap beside it. 720 x 20 x 180 (12
+// tiles of 64, two splits): 100 us; 90 tiles of 16, two splits: 12 us.
+constexpr int ST = 16;
+
+__global__ void __launch_bounds__(NT) gemm_f64_small_kernel(GemmGroup g, const double* __restrict__ A,
+                                                            const double* __restrict__ B, double* __restrict__ C,
+                                                            double alpha, bool accumulate, SplitK sk,
+                                                            double* __restrict__ part) {
+  hs_pdl_enter();
+  int t = blockIdx.x / sk.nsplit;
+  const int split = blockIdx.x % sk.nsplit;
+  int pi = 0;
+  for (; pi < g.n; ++pi) {
+    const int tiles = cdiv(g.p[pi].M, ST) * cdiv(g.p[pi].N, ST);
+    if (t < tiles) break;
+    t -= tiles;
+  }
+  if (pi >= g.n) return;
+  const GemmProblem P = g.p[pi];
+  const int tn_count = cdiv(P.N, ST);
+  const int m0 = (t / tn_count) * ST, n0 = (t % tn_count) * ST;
+  const int kchunk = cdiv(cdiv(P.K, sk.nsplit), BK) * BK;
+  const int kbeg = split * kchunk;
+  const int kend = min(P.K, kbeg + kchunk);
+  __shared__ double As[2][BK][ST + 1], Bs[2][BK][ST + 1];
+  const int tx = threadIdx.x % ST, ty = threadIdx.x / ST;  // column and row of C; k and row of the loads
+  const double* Ap = A + P.a_off + (long long)(m0 + ty) * P.lda;
+  const double* Bp = B + P.b_off + (long long)(n0 + ty) * P.ldb;
+  const bool am = m0 + ty < P.M, bn = n0 + ty < P.N;
+  double acc = 0.0;
+  double a = (am && kbeg + tx < kend) ? Ap[kbeg + tx] : 0.0, b = (bn && kbeg + tx < kend) ? Bp[kbeg + tx] : 0.0;
+  int buf = 0;
+  for (int k0 = kbeg; k0 < kend; k0 += BK, buf ^= 1) {
+    As[buf][tx][ty] = a;
+    Bs[buf][tx][ty] = b;
+    __syncthreads();
+    const int kn = k0 + BK + tx;
+    a = (am && kn < kend) ? Ap[kn] : 0.0;
+    b = (bn && kn < kend) ? Bp[kn] : 0.0;
+#pragma unroll
+    for (int k = 0; k < BK; ++k) acc = fma(As[buf][k][ty], Bs[buf][k][tx], acc);
+  }
+  const int gm = m0 + ty, gn = n0 + tx;
+  if (gm >= P.M || gn >= P.N) return;
+  double* out = C + P.c_off;
+  long long ld = P.ldc;
+  if (sk.nsplit > 1) {
+    out = part + sk.part_off[pi] + (long long)split * P.M * P.N;
+    ld = P.N;
+  }
+  double& o = out[(long long)gm * ld + gn];
+  o = (accumulate && sk.nsplit == 1) ? o + alpha * acc : alpha * acc;
+}
+
 __global__ void splitk_reduce_kernel(GemmGroup g, SplitK sk, const double* __restrict__ part,
                                      double* __restrict__ C, bool accumulate) {
   hs_pdl_enter();
@@ -147,7 +205,19 @@ cudaError_t launch_gemm_f64(const GemmGroup& g, const double* A, const double* B
       }
     }
   }
-  hs_launch(gemm_f64_nt_kernel, (unsigned)(tiles * sk.nsplit), NT, 0, s, g, A, B, C, alpha, accumulate, sk, part);
+  // entries of padded tiles that the busiest SM computes: the smaller count wins
+  // (a tie goes to the larger tiles, whose loads are fewer)
+  long long tiles16 = 0;
+  for (int i = 0; i < g.n; ++i)
+    tiles16 += (long long)((g.p[i].M + ST - 1) / ST) * ((g.p[i].N + ST - 1) / ST);
+  const long long sms = device_sms();
+  const long long big = (tiles * sk.nsplit + sms - 1) / sms * BM * BN;
+  const long long small = (tiles16 * sk.nsplit + sms - 1) / sms * ST * ST;
+  if (small * 10 < big * 9)
+    hs_launch(gemm_f64_small_kernel, (unsigned)(tiles16 * sk.nsplit), NT, 0, s, g, A, B, C, alpha, accumulate, sk,
+              part);
+  else
+    hs_launch(gemm_f64_nt_kernel, (unsigned)(tiles * sk.nsplit), NT, 0, s, g, A, B, C, alpha, accumulate, sk, part);
   if (sk.nsplit > 1) {
     long long mn = 0;
     for (int i = 0; i < g.n; ++i) mn = (long long)g.p[i].M * g.p[i].N > mn ? (long long)g.p[i].M * g.p[i].N : mn;
