@@ -1,12 +1,24 @@
 // Observables of a converged C4v environment (arXiv 2410.11596 Sec. III.A):
 // the two-site reduced density matrix of a bond and the one-site environment
-// eps of Eq. (4). Both are evaluated once per environment, in FP64, as a chain
+// eps of Eq. (4), and the adjoint of the density matrix with the environment
+// held fixed. Both are evaluated once per environment, in FP64, as a chain
 // of permutes and GEMMs over the environment expanded to the plain combined
 // basis; they need the individual bra and ket tensors, which carry no Z2
 // symmetry (Sec. II.B).
 //
 // Networks (C corner, T edge, * open site):
 //   rho:  C T T C / T * * T / C T T C        eps:  C T C / T * T / C T C
+//
+// Order of the contractions (chi = c, q = D^2). The half network of a site
+// is its ring V[x0, e, k0, k1] (corners and two edges), the site's ket tensor
+// over the ket halves of k0 and k1, its bra tensor over the bra halves, and the
+// third edge over (e, k2):
+//   2 c^2 d D^6 (1 + d) + 2 c^3 d^2 q^2 operations and arrays of at most c^2 d^2 q^2
+// entries. Joining the third edge to the ring first and contracting the open
+// double layer as one q^3 index took 2 c^3 q^3 + 2 c^2 d^2 q^4 operations and
+// two arrays of c^2 q^3 (D = 6, c = 144: 836 against 94 GFLOP for both sites,
+// 15.5 against 2.6 GB). eps joins two half rings over both of their boundary
+// bonds, 4 c^3 q^2 + 2 c^2 q^4 operations instead of 2 c^3 q^3 + 2 c^2 q^4.
 #include "hs_ctx.cuh"
 
 using namespace hs;
@@ -89,9 +101,16 @@ __global__ void open_double_layer_vjp_kernel(const double* __restrict__ daoL, co
   }
 }
 
+// Entry (s1, s1', s2, s2') of rho4 from its partial sums, added in order.
+__device__ __forceinline__ double rho4_sum(const double* __restrict__ part, int e, int np) {
+  double v = 0.0;
+  for (int i = 0; i < np; ++i) v += part[(long long)e * np + i];
+  return v;
+}
+
 // rho[(s1 s2), (s1' s2')] = rho4[s1, s1', s2, s2']; mirror the upper triangle
 // when requested; tr[0] = Tr rho, tr[1] = Tr(rho h).
-__global__ void finish_rho_kernel(const double* __restrict__ rho4, int d, bool mirror,
+__global__ void finish_rho_kernel(const double* __restrict__ part, int np, int d, bool mirror,
                                   const double* __restrict__ h, double* __restrict__ rho,
                                   double* __restrict__ tr) {
   hs_pdl_enter();
@@ -104,7 +123,7 @@ __global__ void finish_rho_kernel(const double* __restrict__ rho4, int d, bool m
       J = t;
     }
     const int s1 = I / d, s2 = I % d, t1 = J / d, t2 = J % d;
-    rho[e] = rho4[((s1 * d + t1) * d + s2) * d + t2];
+    rho[e] = rho4_sum(part, ((s1 * d + t1) * d + s2) * d + t2, np);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -234,18 +253,11 @@ unsigned grid_for(long long n) {
   return (unsigned)g;
 }
 
-// A dense tensor with up to 4 groups of legs as an all-even Z2 matrix.
-Z2Mat dense(std::initializer_list<long long> dims) {
+// A dense tensor with its row and column legs as an all-even Z2 matrix.
+Z2Mat dense(std::initializer_list<long long> rows, std::initializer_list<long long> cols) {
   Fused r = fused0(), c = fused0();
-  const int n = (int)dims.size();
-  int i = 0;
-  for (long long v : dims) {
-    if (i < n - 1)
-      r.leg[r.k++] = make_sect((int)v, 0);
-    else
-      c.leg[c.k++] = make_sect((int)v, 0);
-    ++i;
-  }
+  for (long long v : rows) r.leg[r.k++] = make_sect((int)v, 0);
+  for (long long v : cols) c.leg[c.k++] = make_sect((int)v, 0);
   return mat(r, c);
 }
 
@@ -261,46 +273,9 @@ GemmGroup dense_gemm(long long M, long long N, long long K) {
   return g;
 }
 
-// Complex A (interleaved complex128): open double layer with planar output
-//   out[(s, s', m) | (k0, k1, k2)] = A[s, kets] conj(A[s', bras]),
-// where (m, k0, k1, k2) are the legs legs[0..3] (0 u, 1 l, 2 d, 3 r) and each
-// combined index is x = ket + D * bra.
-__global__ void open_double_layer_c_kernel(const double* __restrict__ A, int d, int D, int4 legs,
-                                           double* __restrict__ re, double* __restrict__ im) {
-  hs_pdl_enter();
-  const int q = D * D;
-  const long long total = (long long)d * d * q * q * q * q;
-  const long long D4 = (long long)D * D * D * D;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    long long r = e;
-    int x[4];
-    const int x2 = (int)(r % q);
-    r /= q;
-    const int x1 = (int)(r % q);
-    r /= q;
-    const int x0 = (int)(r % q);
-    r /= q;
-    const int xm = (int)(r % q);
-    r /= q;
-    const int sb = (int)(r % d);
-    const int sk = (int)(r / d);
-    x[legs.x] = xm;
-    x[legs.y] = x0;
-    x[legs.z] = x1;
-    x[legs.w] = x2;
-    const long long ik = (((long long)(x[0] % D) * D + x[1] % D) * D + x[2] % D) * D + x[3] % D;
-    const long long ib = (((long long)(x[0] / D) * D + x[1] / D) * D + x[2] / D) * D + x[3] / D;
-    const double kr = A[2 * (sk * D4 + ik)], ki = A[2 * (sk * D4 + ik) + 1];
-    const double br = A[2 * (sb * D4 + ib)], bi = A[2 * (sb * D4 + ib) + 1];
-    re[e] = kr * br + ki * bi;
-    im[e] = ki * br - kr * bi;
-  }
-}
-
 // Complex rho[(s1 s2), (s1' s2')] = rho4[s1, s1', s2, s2'] (planar in,
 // interleaved out); tr[0..1] = Tr rho, tr[2..3] = Tr(rho h) for real h.
-__global__ void finish_rho_c_kernel(const double* __restrict__ re4, const double* __restrict__ im4, int d,
+__global__ void finish_rho_c_kernel(const double* __restrict__ re4, const double* __restrict__ im4, int np, int d,
                                     const double* __restrict__ h, double* __restrict__ rho, double* __restrict__ tr) {
   hs_pdl_enter();
   const int n = d * d;
@@ -308,8 +283,8 @@ __global__ void finish_rho_c_kernel(const double* __restrict__ re4, const double
     const int I = e / n, J = e % n;
     const int s1 = I / d, s2 = I % d, t1 = J / d, t2 = J % d;
     const int src = ((s1 * d + t1) * d + s2) * d + t2;
-    rho[2 * e] = re4[src];
-    rho[2 * e + 1] = im4[src];
+    rho[2 * e] = rho4_sum(re4, src, np);
+    rho[2 * e + 1] = rho4_sum(im4, src, np);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -330,307 +305,473 @@ __global__ void finish_rho_c_kernel(const double* __restrict__ re4, const double
   }
 }
 
+// ---- kernels of the two-site network ------------------------------------------
+//
+// A half network L or R is [(x0, s, mk, s', mb) | x4]: boundary bond, ket and
+// bra physical index with the ket and bra halves of the bond m between the
+// sites, the other boundary bond. Complex ones are planar.
+
+constexpr int kRhoParts = 64;
+
+// Partial sums of rho4[s1, s1', s2, s2'] = sum_{x0, mk, mb, x4} L R: part[pair][i]
+// from every kRhoParts-th (x0, mk, mb). Bound by the FP64 pipe (d^4 c^2 q FMAs,
+// 23 us at D = 6, c = 144), with the operands read from L2; a 4 x 4 GEMM over
+// c^2 q would leave 255 of 256 tile entries idle.
+__global__ void __launch_bounds__(128) rho4_kernel(const double* __restrict__ Lr, const double* __restrict__ Li,
+                                                   const double* __restrict__ Rr, const double* __restrict__ Ri, int d,
+                                                   int D, int chi, double* __restrict__ part_re,
+                                                   double* __restrict__ part_im) {
+  hs_pdl_enter();
+  const int pair = blockIdx.x, s2b = pair % d, s2 = pair / d % d, s1b = pair / d / d % d, s1 = pair / d / d / d;
+  double re = 0.0, im = 0.0;
+  for (int u = blockIdx.y; u < chi * D * D; u += kRhoParts) {
+    const int mb = u % D, mk = u / D % D, x0 = u / D / D;
+    const long long lo = (((((long long)x0 * d + s1) * D + mk) * d + s1b) * D + mb) * chi;
+    const long long ro = (((((long long)x0 * d + s2) * D + mk) * d + s2b) * D + mb) * chi;
+    for (int x = threadIdx.x; x < chi; x += blockDim.x) {
+      re += Lr[lo + x] * Rr[ro + x];
+      if (Li) {
+        re -= Li[lo + x] * Ri[ro + x];
+        im += Lr[lo + x] * Ri[ro + x] + Li[lo + x] * Rr[ro + x];
+      }
+    }
+  }
+  __shared__ double red[2][4];
+  for (int o = 16; o > 0; o >>= 1) {
+    re += __shfl_down_sync(0xffffffffu, re, o);
+    im += __shfl_down_sync(0xffffffffu, im, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x / 32] = re;
+    red[1][threadIdx.x / 32] = im;
+  }
+  __syncthreads();
+  if (threadIdx.x < (Li ? 2 : 1))
+    (threadIdx.x ? part_im : part_re)[(long long)pair * kRhoParts + blockIdx.y] =
+        (red[threadIdx.x][0] + red[threadIdx.x][1]) + (red[threadIdx.x][2] + red[threadIdx.x][3]);
+}
+
+// Cotangent of one half network from that of rho and the other half:
+//   out[.., s, .., s', ..] = sum_{o, o'} g conj(in[.., o, .., o', ..]),
+// g = drho[(s o), (s' o')] for the left half, drho[(o s), (o' s')] for the right
+// one (drho real, or interleaved complex). One thread per (x0, mk, mb, x4).
+__global__ void half_adjoint_kernel(const double* __restrict__ drho, const double* __restrict__ in_re,
+                                    const double* __restrict__ in_im, int d, int D, int chi, bool left,
+                                    double* __restrict__ out_re, double* __restrict__ out_im) {
+  hs_pdl_enter();
+  const long long total = (long long)chi * D * D * chi;
+  const int n = d * d;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int x4 = (int)(e % chi);
+    const long long u = e / chi;
+    const int mb = (int)(u % D), mk = (int)(u / D % D);
+    const long long x0 = u / D / D;
+    auto at = [&](int s, int sb) { return (((((x0 * d + s) * D + mk) * d + sb) * D + mb) * chi + x4); };
+    for (int s = 0; s < d; ++s)
+      for (int sb = 0; sb < d; ++sb) {
+        double re = 0.0, im = 0.0;
+        for (int o = 0; o < d; ++o)
+          for (int ob = 0; ob < d; ++ob) {
+            const int I = left ? s * d + o : o * d + s, J = left ? sb * d + ob : ob * d + sb;
+            const long long src = at(o, ob);
+            if (!in_im) {
+              re += drho[I * n + J] * in_re[src];
+            } else {
+              const double gr = drho[2 * (I * n + J)], gi = drho[2 * (I * n + J) + 1];
+              re += gr * in_re[src] + gi * in_im[src];
+              im += gi * in_re[src] - gr * in_im[src];
+            }
+          }
+        out_re[at(s, sb)] = re;
+        if (in_im) out_im[at(s, sb)] = im;
+      }
+  }
+}
+
+// Which legs of A[s, u, l, d, r] (1..4) are a site's m, k2, k0 and k1.
+struct SiteLegs {
+  int m, k2, k0, k1;
+};
+
+// Position of (s, m, k2, k0, k1) in A[s, u, l, d, r].
+__device__ __forceinline__ int a_index(int s, int m, int k2, int k0, int k1, SiteLegs g, int D) {
+  int x[5];
+  x[0] = s;
+  x[g.m] = m;
+  x[g.k2] = k2;
+  x[g.k0] = k0;
+  x[g.k1] = k1;
+  return (((x[0] * D + x[1]) * D + x[2]) * D + x[3]) * D + x[4];
+}
+
+// The cotangent Q[(s, mk, s', mb, k2k, k2b) | (k0b, k0k, k1b, k1k)] of a site's open
+// double layer a = A_ket conj(A_bra), contracted with A row by row (one block
+// per row of q^2 contiguous entries, so that Q is read once):
+//   pk[row][k0k, k1k] = sum_{k0b, k1b} Q A[s', bra],
+//   pb[row][k0b, k1b] = sum_{k0k, k1k} conj(Q) A[s, ket].
+// site_sum_kernel adds them up. Bound by reading Q (54 MB at D = 6).
+__global__ void __launch_bounds__(64) site_adjoint_kernel(const double* __restrict__ Qr, const double* __restrict__ Qi,
+                                                          const double* __restrict__ A, int d, int D, SiteLegs g,
+                                                          bool staged, double* __restrict__ pk,
+                                                          double* __restrict__ pb) {
+  hs_pdl_enter();
+  extern __shared__ double sh[];
+  const int q = D * D, cx = Qi ? 2 : 1;
+  double* ket = sh;  // A[s, ket] over (k0, k1), A[s', bra]
+  double* bra = ket + cx * q;
+  double* row = bra + cx * q;  // the row's q^2 entries (complex: re, then im), when they fit
+  long long r = blockIdx.x;
+  const int k2b = (int)(r % D), k2k = (int)(r / D % D), mb = (int)(r / q % D), sb = (int)(r / q / D % d),
+            mk = (int)(r / q / D / d % D), s = (int)(r / q / D / d / D);
+  const long long base = (long long)blockIdx.x * q * q;
+  if (staged)
+    for (int i = threadIdx.x; i < q * q; i += blockDim.x) {
+      row[i] = Qr[base + i];
+      if (cx == 2) row[q * q + i] = Qi[base + i];
+    }
+  const double* qr = staged ? row : Qr + base;
+  const double* qi = staged ? row + q * q : Qi + base;
+  for (int i = threadIdx.x; i < q; i += blockDim.x) {
+    const int ik = a_index(s, mk, k2k, i / D, i % D, g, D), ib = a_index(sb, mb, k2b, i / D, i % D, g, D);
+    for (int c = 0; c < cx; ++c) {
+      ket[c * q + i] = A[cx * ik + c];
+      bra[c * q + i] = A[cx * ib + c];
+    }
+  }
+  __syncthreads();
+  for (int o = threadIdx.x; o < 2 * q; o += blockDim.x) {
+    const bool is_ket = o < q;
+    const int i0 = o % q / D, i1 = o % D;
+    double re = 0.0, im = 0.0;
+    for (int j = 0; j < q; ++j) {
+      const int j0 = j / D, j1 = j % D;
+      const int at = is_ket ? ((j0 * D + i0) * D + j1) * D + i1 : ((i0 * D + j0) * D + i1) * D + j1;
+      const double* a = is_ket ? bra : ket;
+      if (cx == 1) {
+        re += qr[at] * a[j];
+      } else {
+        const double gr = qr[at], gi = is_ket ? qi[at] : -qi[at];
+        re += gr * a[j] - gi * a[q + j];
+        im += gr * a[q + j] + gi * a[j];
+      }
+    }
+    double* out = (is_ket ? pk : pb) + ((long long)blockIdx.x * q + o % q) * cx;
+    out[0] = re;
+    if (cx == 2) out[1] = im;
+  }
+}
+
+// dA (= or +=) the sums of pk over (s', mb, k2b) and of pb over (s, mk, k2k).
+__global__ void site_sum_kernel(const double* __restrict__ pk, const double* __restrict__ pb, int d, int D, int cx,
+                                SiteLegs g, bool add, double* __restrict__ dA) {
+  hs_pdl_enter();
+  const int q = D * D, nS = d * D;
+  const long long nA = (long long)d * q * q;
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nA * cx;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int c = (int)(e % cx);
+    const int i = (int)(e / cx);
+    const int k1 = i % D, k0 = i / D % D, k2 = i / q % D, m = i / q / D % D, s = i / q / q;
+    const int S = s * D + m;
+    double v = 0.0;
+    for (int T = 0; T < nS; ++T)
+      for (int o = 0; o < D; ++o) {
+        const long long rk = (((long long)S * nS + T) * D + k2) * D + o;  // this element as the ket
+        const long long rb = (((long long)T * nS + S) * D + o) * D + k2;  // as the bra
+        v += pk[(rk * q + k0 * D + k1) * cx + c] + pb[(rb * q + k0 * D + k1) * cx + c];
+      }
+    const long long a = (long long)a_index(s, m, k2, k0, k1, g, D) * cx + c;
+    dA[a] = add ? dA[a] + v : v;
+  }
+}
+
+// ---- the chains -------------------------------------------------------------------
+
+// A real array, or a complex one as planar real and imaginary parts.
 struct ZBuf {
   double* re;
   double* im;
 };
 
-// planar buffer pair i (0 <= i < 20) of the context, at least n doubles each
-ZBuf zbuf(hs_ctx ctx, int i, long long n) {
-  if (i < 0 || 2 * i + 1 >= (int)(sizeof(ctx->zr) / sizeof(ctx->zr[0]))) return {nullptr, nullptr};
-  if (ctx->zr[2 * i].ensure(n * 8) != HS_OK || ctx->zr[2 * i + 1].ensure(n * 8) != HS_OK) return {nullptr, nullptr};
-  return {ctx->zr[2 * i].d(), ctx->zr[2 * i + 1].d()};
-}
+// One observable's evaluation: real or complex arithmetic on the context's buffers.
+struct Obs {
+  hs_ctx ctx;
+  bool cx;
+  hs_gemm_backend be;
+  long long c, q, d, D;
 
-// complex C = A B^T (or A conj(B)^T) from planar parts
-hs_status zgemm(hs_ctx ctx, const GemmGroup& g, ZBuf A, ZBuf B, ZBuf C, bool conj_b = false) {
-  return zgemm_f64(ctx, g, A.re, A.im, B.re, B.im, C.re, C.im, conj_b);
-}
-
-// dA of a complex A from the cotangents g1, g2 of the two open double layers
-// (planar; layouts of open_double_layer_c_kernel with legs1 / legs2). For a
-// real energy the cotangent convention is g = dE/dRe + i dE/dIm; a site's
-// a[s, s', ...] = A[s, ket] conj(A[s', bra]) gives
-//   dA[p, mine] += g[p, s', (mine as ket, other as bra)] A[s', other]
-//                + conj(g[s, p, (other as ket, mine as bra)]) A[s, other].
-__global__ void open_double_layer_c_vjp_kernel(const double* __restrict__ g1r, const double* __restrict__ g1i,
-                                               int4 legs1, const double* __restrict__ g2r,
-                                               const double* __restrict__ g2i, int4 legs2,
-                                               const double* __restrict__ A, int d, int D, double* __restrict__ dA) {
-  hs_pdl_enter();
-  const int q = D * D;
-  const long long D4 = (long long)D * D * D * D;
-  const long long nA = d * D4;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nA;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int p = (int)(e / D4);
-    long long t = e % D4;
-    int mine[4];
-    mine[3] = (int)(t % D);
-    t /= D;
-    mine[2] = (int)(t % D);
-    t /= D;
-    mine[1] = (int)(t % D);
-    mine[0] = (int)(t / D);
-    double ar = 0.0, ai = 0.0;
-    for (int s2 = 0; s2 < d; ++s2)
-      for (long long o = 0; o < D4; ++o) {
-        long long oo = o;
-        int oth[4];
-        oth[3] = (int)(oo % D);
-        oo /= D;
-        oth[2] = (int)(oo % D);
-        oo /= D;
-        oth[1] = (int)(oo % D);
-        oth[0] = (int)(oo / D);
-        int xk[4], xb[4];
-        for (int l = 0; l < 4; ++l) {
-          xk[l] = mine[l] + D * oth[l];  // this element as the ket factor
-          xb[l] = oth[l] + D * mine[l];  // this element as the bra factor
-        }
-        const double Or = A[2 * (s2 * D4 + o)], Oi = A[2 * (s2 * D4 + o) + 1];
-        for (int site = 0; site < 2; ++site) {
-          const int4 L = site ? legs2 : legs1;
-          const double* gr = site ? g2r : g1r;
-          const double* gi = site ? g2i : g1i;
-          const long long ik =
-              ((((((long long)p * d + s2) * q + xk[L.x]) * q + xk[L.y]) * q + xk[L.z]) * q + xk[L.w]);
-          const long long ib =
-              ((((((long long)s2 * d + p) * q + xb[L.x]) * q + xb[L.y]) * q + xb[L.z]) * q + xb[L.w]);
-          // g_ket * A_other + conj(g_bra) * A_other
-          const double cr = gr[ik] + gr[ib], ci = gi[ik] - gi[ib];
-          ar += cr * Or - ci * Oi;
-          ai += cr * Oi + ci * Or;
-        }
-      }
-    dA[2 * e] = ar;
-    dA[2 * e + 1] = ai;
+  // buffer i (0 <= i < 20), at least n entries
+  hs_status buf(int i, long long n, ZBuf* z) const {
+    HS_TRY(ctx->zr[2 * i].ensure(n * 8));
+    if (cx) HS_TRY(ctx->zr[2 * i + 1].ensure(n * 8));
+    *z = {ctx->zr[2 * i].d(), cx ? ctx->zr[2 * i + 1].d() : nullptr};
+    return HS_OK;
   }
+  // C[M | N] = A[M | K] B[N | K]^T (or conj(B))
+  hs_status mul(long long M, long long N, long long K, ZBuf A, ZBuf B, ZBuf C, bool conj_b = false) const {
+    const GemmGroup g = dense_gemm(M, N, K);
+    if (cx) return zgemm_f64(ctx, g, A.re, A.im, B.re, B.im, C.re, C.im, conj_b);
+    return gemm(ctx, be, g, A.re, B.re, C.re);
+  }
+  hs_status perm(const Z2Mat& in, const Z2Mat& out, std::initializer_list<int> p, ZBuf src, ZBuf dst) const {
+    HS_TRY(permute(ctx, in, out, p, src.re, dst.re));
+    return cx ? permute(ctx, in, out, p, src.im, dst.im) : HS_OK;
+  }
+  // interleaved complex -> planar
+  hs_status planar(const double* src, long long n, ZBuf dst, DBuf& tmp) const {
+    HS_TRY(tmp.ensure(2 * n * 8));
+    HS_TRY(permute(ctx, dense({n}, {2}), dense({2}, {n}), {1, 0}, src, tmp.d()));
+    HS_CUDA(cudaMemcpyAsync(dst.re, tmp.d(), n * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+    HS_CUDA(cudaMemcpyAsync(dst.im, tmp.d() + n, n * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+    return HS_OK;
+  }
+};
+
+// Buffers kept between the steps of a chain; the others are scratch.
+enum { bT = 0, bH, bV, bA, bL, bR, bPart, bScratch };
+
+Obs make_obs(hs_ctx ctx, const hs_env* env, int d, int D) {
+  return {ctx, env->dtype == HS_C128, env->gemm_backend, (long long)env->chi_even + env->chi_odd, (long long)D * D, d,
+          D};
 }
 
-hs_status zpermute(hs_ctx ctx, const Z2Mat& in, const Z2Mat& out, std::initializer_list<int> perm, ZBuf src,
-                   ZBuf dst) {
-  HS_TRY(permute(ctx, in, out, perm, src.re, dst.re));
-  return permute(ctx, in, out, perm, src.im, dst.im);
+// The environment in the plain combined basis: T[(a, x) | b] (bT) and the half
+// ring H[(a, x) | b] = C[a, c] T[c, x, e] C[e, b] (bH).
+hs_status half_ring(const Obs& o, const hs_env* env, int D) {
+  hs_ctx ctx = o.ctx;
+  const long long c = o.c, q = o.q, c2 = c * c, cqc = c * q * c;
+  ZBuf C, T, Ct, Tq, H1, H;
+  HS_TRY(o.buf(bT, cqc, &T));
+  HS_TRY(o.buf(bH, cqc, &H));
+  HS_TRY(o.buf(bScratch, c2, &C));
+  HS_TRY(o.buf(bScratch + 1, c2, &Ct));
+  HS_TRY(o.buf(bScratch + 2, cqc, &Tq));
+  HS_TRY(o.buf(bScratch + 3, cqc, &H1));
+  if (!o.cx) {
+    HS_CUDA(launch_env_to_dense(env->C, env->T, D, env->chi_even, env->chi_odd, env->basis == HS_BASIS_HERMITIAN, C.re,
+                                T.re, ctx->stream));
+  } else if (env->basis == HS_BASIS_DENSE) {
+    // a complex environment of the plain basis is stored dense already
+    HS_TRY(o.planar(env->C, c2, C, ctx->r[2]));
+    HS_TRY(o.planar(env->T, cqc, T, ctx->r[2]));
+  } else {
+    HS_TRY(ctx->r[0].ensure(2 * c2 * 8));
+    HS_TRY(ctx->r[1].ensure(2 * cqc * 8));
+    HS_CUDA(launch_env_to_dense_graded(env->C, env->T, D, env->chi_even, env->chi_odd, ctx->r[0].d(), ctx->r[1].d(),
+                                       ctx->stream));
+    HS_TRY(o.planar(ctx->r[0].d(), c2, C, ctx->r[2]));
+    HS_TRY(o.planar(ctx->r[1].d(), cqc, T, ctx->r[2]));
+  }
+  HS_TRY(o.perm(dense({c}, {c}), dense({c}, {c}), {1, 0}, C, Ct));
+  HS_TRY(o.perm(dense({c, q}, {c}), dense({q, c}, {c}), {1, 2, 0}, T, Tq));  // Tq[(x, e) | c]
+  HS_TRY(o.mul(c, q * c, c, C, Tq, H1));                                      // H1[a | (x, e)]
+  return o.mul(c * q, c, c, H1, Ct, H);                                       // H[(a, x) | b]
+}
+
+// eps[u, l, d, r] (Eq. (4)) from two half rings joined over both boundary bonds.
+//   real:    up[t, u, l, t'..] E[t, u, b] T[t, l, t'] and T[b, r, b'] E[t', d, b'] over (b, t')
+//   complex: H[a, u, b] T[b, r, b'] and H[b', d, a'] T[a', l, a] over (a, b') (clockwise ring)
+hs_status one_site_chain(hs_ctx ctx, const hs_env* env, int d, int D, double* eps) {
+  const Obs o = make_obs(ctx, env, d, D);
+  HS_TRY(half_ring(o, env, D));
+  const long long c = o.c, q = o.q, n = c * c * q * q, q4 = q * q * q * q;
+  ZBuf T, H, W1, W2, U, W, E, x1, x2;
+  HS_TRY(o.buf(bT, c * q * c, &T));
+  HS_TRY(o.buf(bH, c * q * c, &H));
+  HS_TRY(o.buf(bScratch, n, &W1));
+  HS_TRY(o.buf(bScratch + 1, n, &U));
+  HS_TRY(o.buf(bScratch + 2, n, &W2));
+  HS_TRY(o.buf(bScratch + 3, n, &W));
+  HS_TRY(o.buf(bScratch + 4, c * q * c, &x1));
+  HS_TRY(o.buf(bScratch + 5, c * q * c, &x2));
+  HS_TRY(o.buf(bScratch + 6, q4, &E));
+  const Z2Mat edge = dense({c, q}, {c}), rev = dense({c, q}, {c});
+  if (!o.cx) {
+    HS_TRY(o.perm(edge, rev, {2, 1, 0}, H, x1));                                                    // [(b, u) | t]
+    HS_TRY(o.perm(edge, rev, {2, 1, 0}, T, x2));                                                    // [(t', l) | t]
+    HS_TRY(o.mul(c * q, c * q, c, x1, x2, W1));                                                     // [(b, u) | (t', l)]
+    HS_TRY(o.perm(dense({c, q}, {c, q}), dense({q, q}, {c, c}), {1, 3, 0, 2}, W1, U));              // [(u, l) | (b, t')]
+    HS_TRY(o.mul(c * q, c * q, c, T, H, W2));                                                       // [(b, r) | (t', d)]
+    HS_TRY(o.perm(dense({c, q}, {c, q}), dense({q, q}, {c, c}), {3, 1, 0, 2}, W2, W));              // [(d, r) | (b, t')]
+    return gemm(ctx, o.be, dense_gemm(q * q, q * q, c * c), U.re, W.re, eps);                       // [(u, l) | (d, r)]
+  }
+  HS_TRY(o.perm(edge, rev, {2, 1, 0}, T, x1));                                                      // [(b', r) | b]
+  HS_TRY(o.mul(c * q, c * q, c, H, x1, W1));                                                        // [(a, u) | (b', r)]
+  HS_TRY(o.perm(dense({c, q}, {c, q}), dense({q, q}, {c, c}), {1, 3, 0, 2}, W1, U));                // [(u, r) | (a, b')]
+  HS_TRY(o.perm(edge, rev, {2, 1, 0}, T, x1));                                                      // [(a, l) | a']
+  HS_TRY(o.mul(c * q, c * q, c, x1, H, W2));                                                        // [(a, l) | (b', d)]
+  HS_TRY(o.perm(dense({c, q}, {c, q}), dense({q, q}, {c, c}), {1, 3, 0, 2}, W2, W));                // [(l, d) | (a, b')]
+  HS_TRY(o.mul(q * q, q * q, c * c, U, W, E));                                                      // [(u, r) | (l, d)]
+  ZBuf Eo;
+  HS_TRY(ctx->r[2].ensure(2 * q4 * 8));
+  Eo = {ctx->r[2].d(), ctx->r[2].d() + q4};
+  HS_TRY(o.perm(dense({q, q}, {q, q}), dense({q, q}, {q, q}), {0, 2, 3, 1}, E, Eo));                // u, l, d, r
+  return permute(ctx, dense({2}, {q4}), dense({q4}, {2}), {1, 0}, ctx->r[2].d(), eps);
+}
+
+// The legs of the two sites (index into A[s, u, l, d, r]); m joins the sites.
+//   real:    V over the site's outer leg, then up; the bottom edge closes k2 = down
+//   complex: left chain down, outer, up; right chain up, outer, down (clockwise)
+SiteLegs site_legs(bool cx, bool left) {
+  if (!cx) return left ? SiteLegs{4, 3, 2, 1} : SiteLegs{2, 3, 4, 1};
+  return left ? SiteLegs{4, 1, 3, 2} : SiteLegs{2, 3, 1, 4};
+}
+
+// A site's half network out[(x0, S, S') | x4], S = (s, m): Xp[(x0, e, k0b, k1b) | (k0k, k1k)]
+// with the ket tensor, the bra tensor and the edge T[e, k2, x4].
+hs_status site_half(const Obs& o, ZBuf Xp, const SiteLegs& g, ZBuf out) {
+  const long long c = o.c, D = o.D, q = o.q, S = o.d * D;
+  ZBuf A, AP, T, TB, Y1, Y1p, Y2, Xf;
+  const long long n1 = c * c * q * S * D, n2 = c * c * S * D * S * D;
+  HS_TRY(o.buf(bA, S * D * q, &A));
+  HS_TRY(o.buf(bT, c * q * c, &T));
+  HS_TRY(o.buf(bScratch + 1, S * D * q, &AP));
+  HS_TRY(o.buf(bScratch + 2, c * q * c, &TB));
+  HS_TRY(o.buf(bScratch + 3, n2 > n1 ? n2 : n1, &Y1));
+  HS_TRY(o.buf(bScratch + 4, n2 > n1 ? n2 : n1, &Y1p));
+  Y2 = Y1;
+  Xf = Y1p;
+  HS_TRY(o.perm(dense({o.d, D, D, D}, {D}), dense({o.d, D, D}, {D, D}), {0, g.m, g.k2, g.k0, g.k1}, A, AP));
+  HS_TRY(o.perm(dense({c, D, D}, {c}), dense({c}, {c, D, D}), {3, 0, 2, 1}, T, TB));              // [x4 | (e, k2k, k2b)]
+  HS_TRY(o.mul(c * c * q, S * D, q, Xp, AP, Y1));                                                  // [(x0, e, k0b, k1b) | (S, k2k)]
+  HS_TRY(o.perm(dense({c * c, q}, {S * D}), dense({c * c, S * D}, {q}), {0, 2, 1}, Y1, Y1p));      // [(x0, e, S, k2k) | (k0b, k1b)]
+  HS_TRY(o.mul(c * c * S * D, S * D, q, Y1p, AP, Y2, true));                                       // [(x0, e, S, k2k) | (S', k2b)]
+  HS_TRY(o.perm(dense({c, c, S, D}, {S, D}), dense({c, S, S}, {c, D, D}), {0, 2, 4, 1, 3, 5}, Y2, Xf));
+  return o.mul(c * S * S, c, c * q, Xf, TB, out);
+}
+
+// Forward chain of the two-site network: leaves T (bT), the ring V (bV, [(e, k0) | (x0, k1)]
+// real, [(x0, k0) | (e, k1)] complex), the tensor A (bA), the half networks of
+// the left site L[(x0, S, S') | x4] (bL) and the right one (bR, x0 and x4 those of
+// L), and the partial sums of rho4 (bPart).
+hs_status rdm_chain(hs_ctx ctx, const hs_env* env, const double* A, int d, int D) {
+  const Obs o = make_obs(ctx, env, d, D);
+  HS_TRY(half_ring(o, env, D));
+  const long long c = o.c, q = o.q, nA = (long long)d * q * q, nh = c * c * d * d * q, nx = c * c * q * q;
+  ZBuf T, H, V, Az, L, R, part, Xp, x1, x2;
+  HS_TRY(o.buf(bT, c * q * c, &T));
+  HS_TRY(o.buf(bH, c * q * c, &H));
+  HS_TRY(o.buf(bV, nx, &V));
+  HS_TRY(o.buf(bA, nA, &Az));
+  HS_TRY(o.buf(bL, nh, &L));
+  HS_TRY(o.buf(bR, nh, &R));
+  HS_TRY(o.buf(bPart, (long long)d * d * d * d * kRhoParts, &part));
+  HS_TRY(o.buf(bScratch, nx, &Xp));
+  HS_TRY(o.buf(bScratch + 1, c * q * c, &x1));
+  HS_TRY(o.buf(bScratch + 2, c * q * c, &x2));
+  if (o.cx)
+    HS_TRY(o.planar(A, nA, Az, ctx->r[2]));
+  else
+    HS_CUDA(cudaMemcpyAsync(Az.re, A, nA * 8, cudaMemcpyDeviceToDevice, ctx->stream));
+  const Z2Mat edge = dense({c, q}, {c});
+  const Z2Mat vl = dense({c, D, D}, {c, D, D}), xl = dense({c, c, D, D}, {D, D});
+  if (!o.cx) {
+    // V[b, l, t', u] = E[t, l, b] T[t, u, t']: x0 = t', e = b, k0 = l (r on the right), k1 = u
+    HS_TRY(o.perm(edge, edge, {2, 1, 0}, H, x1));
+    HS_TRY(o.perm(edge, edge, {2, 1, 0}, T, x2));
+    HS_TRY(o.mul(c * q, c * q, c, x1, x2, V));
+    HS_TRY(o.perm(vl, xl, {3, 0, 1, 4, 2, 5}, V, Xp));
+  } else {
+    // V[x0, k0, e, k1] = T[x0, k0, a] H[a, k1, e]
+    HS_TRY(o.perm(edge, edge, {2, 1, 0}, H, x1));
+    HS_TRY(o.mul(c * q, c * q, c, T, x1, V));
+    HS_TRY(o.perm(vl, xl, {0, 3, 1, 4, 2, 5}, V, Xp));
+  }
+  HS_TRY(site_half(o, Xp, site_legs(o.cx, true), L));
+  if (!o.cx) {
+    HS_TRY(site_half(o, Xp, site_legs(false, false), R));
+  } else {
+    // the right chain runs from t to b: exchanged to the left one's bonds
+    ZBuf Rt;
+    HS_TRY(o.buf(bScratch + 5, nh, &Rt));
+    HS_TRY(site_half(o, Xp, site_legs(true, false), Rt));
+    HS_TRY(o.perm(dense({c, (long long)d * d * q}, {c}), dense({c, (long long)d * d * q}, {c}), {2, 1, 0}, Rt, R));
+  }
+  hs_launch(rho4_kernel, dim3((unsigned)(d * d * d * d), kRhoParts), 128, 0, ctx->stream, (const double*)L.re,
+            (const double*)L.im, (const double*)R.re, (const double*)R.im, d, D, (int)c, part.re, part.im);
+  HS_CUDA(cudaGetLastError());
+  ctx->launches += 1;
+  return HS_OK;
+}
+
+// rho and its traces from rdm_chain's partial sums.
+hs_status finish_rdm(hs_ctx ctx, const hs_env* env, int d, int D, const double* h, double* rho, double* tr) {
+  const Obs o = make_obs(ctx, env, d, D);
+  ZBuf part;
+  HS_TRY(o.buf(bPart, (long long)d * d * d * d * kRhoParts, &part));
+  if (o.cx)
+    hs_launch(finish_rho_c_kernel, 1, 256, 0, ctx->stream, (const double*)part.re, (const double*)part.im, kRhoParts, d,
+              h, rho, tr);
+  else
+    hs_launch(finish_rho_kernel, 1, 256, 0, ctx->stream, (const double*)part.re, kRhoParts, d,
+              env->basis == HS_BASIS_HERMITIAN, h, rho, tr);
+  HS_CUDA(cudaGetLastError());
+  ctx->launches += 1;
+  return HS_OK;
+}
+
+// Reverse pass of rdm_chain, which must have run on the same environment and A
+// just before: drho (d^4, real or interleaved complex) -> dA. Per site: the
+// half network's cotangent, through the edge to the ring and the open double
+// layer, Q = dXf conj(V) over the boundary bonds, then A (site_adjoint_kernel).
+hs_status rdm_vjp_after_chain(hs_ctx ctx, const hs_env* env, int d, int D, const double* A, const double* drho,
+                              double* dA_out) {
+  const Obs o = make_obs(ctx, env, d, D);
+  const long long c = o.c, q = o.q, S = (long long)d * D, nh = c * c * S * S, nx = c * c * q * q, nf = c * S * S * c * q,
+                  nq = S * S * q * q * q;
+  ZBuf T, V, half[2], dh, dht, TT, Vt, F, Fp, Q, pp;
+  HS_TRY(o.buf(bT, c * q * c, &T));
+  HS_TRY(o.buf(bV, nx, &V));
+  HS_TRY(o.buf(bL, nh, &half[0]));
+  HS_TRY(o.buf(bR, nh, &half[1]));
+  HS_TRY(o.buf(bScratch, nx, &Vt));
+  HS_TRY(o.buf(bScratch + 2, c * q * c, &TT));
+  HS_TRY(o.buf(bScratch + 3, nf, &F));
+  HS_TRY(o.buf(bScratch + 4, nf, &Fp));
+  HS_TRY(o.buf(bScratch + 5, nh, &dh));
+  HS_TRY(o.buf(bScratch + 6, nq, &Q));
+  HS_TRY(o.buf(bScratch + 7, nh, &dht));
+  const int cx = o.cx ? 2 : 1;
+  const long long rows = S * S * q, npart = rows * q * cx;
+  HS_TRY(ctx->hb[0].ensure(2 * npart * 8));
+  double *pk = ctx->hb[0].d(), *pb = pk + npart;
+  HS_TRY(o.perm(dense({c, D, D}, {c}), dense({c, D, D}, {c}), {0, 2, 1, 3}, T, TT));  // [(e, k2k, k2b) | x4]
+  if (!o.cx)
+    HS_TRY(o.perm(dense({c, q}, {c, q}), dense({q, q}, {c, c}), {1, 3, 2, 0}, V, Vt));  // [(k0, k1) | (x0, e)]
+  else
+    HS_TRY(o.perm(dense({c, q}, {c, q}), dense({q, q}, {c, c}), {1, 3, 0, 2}, V, Vt));
+  size_t sm = (size_t)(cx * (q * q + 2 * q)) * sizeof(double);
+  constexpr size_t kMaxRow = 200 * 1024;
+  const bool staged = sm <= kMaxRow;
+  if (!staged) sm = (size_t)(cx * 2 * q) * sizeof(double);
+  HS_CUDA(ensure_smem_attr(reinterpret_cast<const void*>(site_adjoint_kernel), (int)kMaxRow));
+  for (int site = 0; site < 2; ++site) {
+    const bool left = site == 0;
+    const SiteLegs g = site_legs(o.cx, left);
+    hs_launch(half_adjoint_kernel, grid_for(c * q * c), 256, 0, ctx->stream, drho, (const double*)half[1 - site].re,
+              (const double*)half[1 - site].im, d, D, (int)c, left, dh.re, dh.im);
+    HS_CUDA(cudaGetLastError());
+    ZBuf din = dh;
+    if (o.cx && !left) {  // back to the right chain's own bonds
+      HS_TRY(o.perm(dense({c, S * S}, {c}), dense({c, S * S}, {c}), {2, 1, 0}, dh, dht));
+      din = dht;
+    }
+    HS_TRY(o.mul(c * S * S, c * q, c, din, TT, F, true));  // [(x0, S, S') | (e, k2k, k2b)]
+    HS_TRY(o.perm(dense({c, S, S}, {c, D, D}), dense({S, S, D, D}, {c, c}), {1, 2, 4, 5, 0, 3}, F, Fp));
+    HS_TRY(o.mul(rows, q * q, c * c, Fp, Vt, Q, true));  // [(S, S', k2k, k2b) | (k0, k1)]
+    hs_launch(site_adjoint_kernel, (unsigned)rows, 64, sm, ctx->stream, (const double*)Q.re, (const double*)Q.im, A, d,
+              D, g, staged, pk, pb);
+    HS_CUDA(cudaGetLastError());
+    hs_launch(site_sum_kernel, grid_for((long long)d * q * q * cx), 256, 0, ctx->stream, (const double*)pk,
+              (const double*)pb, d, D, cx, g, !left, dA_out);
+    HS_CUDA(cudaGetLastError());
+    ctx->launches += 3;
+  }
+  return HS_OK;
 }
 
 }  // namespace
-
-// Two-site rho of a complex (graded, oriented) environment: the network of
-// the oracle's clockwise ring, in complex arithmetic on planar FP64 parts.
-// Chain (C, T dense from the graded environment; boundary tensors clockwise):
-//   H[a,x,b] = C[a,c] T[c,x,e] C[e,b]
-//   L[b,d1,l1,u1,t] = T[b,d1,c] H[c,l1,e] T[e,u1,t]  (also the right chain R[t,u2,r2,d2,b])
-//   LB[(b,t)|(s1,s1',m)] = L a1 over (d1,l1,u1); RB[(t,b)|(s2,s2',m)] = L a2 over (u2,r2,d2)
-//   rho4[(s1,s1')|(s2,s2')] = sum_{b,t,m} LB RB
-hs_status rdm_complex(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, hs_rdm_kind kind,
-                      const double* h, double* out, double* tr_out) {
-  cudaStream_t s = ctx->stream;
-  const long long chi = env->chi_even + env->chi_odd, q = (long long)D * D, d2 = (long long)d * d;
-  const long long c2 = chi * chi, cqc = chi * q * chi, c2q2 = c2 * q * q, c2q3 = c2q2 * q;
-  // interleaved dense environment, then planar
-  HS_TRY(ctx->r[0].ensure(2 * c2 * 8));
-  HS_TRY(ctx->r[1].ensure(2 * cqc * 8));
-  if (env->basis == HS_BASIS_DENSE) {
-    // a complex environment of the plain basis is stored dense already
-    HS_CUDA(cudaMemcpyAsync(ctx->r[0].d(), env->C, 2 * c2 * 8, cudaMemcpyDeviceToDevice, s));
-    HS_CUDA(cudaMemcpyAsync(ctx->r[1].d(), env->T, 2 * cqc * 8, cudaMemcpyDeviceToDevice, s));
-  } else {
-    HS_CUDA(launch_env_to_dense_graded(env->C, env->T, D, env->chi_even, env->chi_odd, ctx->r[0].d(), ctx->r[1].d(),
-                                       s));
-  }
-  ZBuf Cz = zbuf(ctx, 0, c2), Tz = zbuf(ctx, 1, cqc), Ctz = zbuf(ctx, 2, c2), Tqz = zbuf(ctx, 3, cqc),
-       H1 = zbuf(ctx, 4, cqc), Hz = zbuf(ctx, 5, cqc), Hq = zbuf(ctx, 6, cqc), L1 = zbuf(ctx, 7, c2q2),
-       L2 = zbuf(ctx, 8, c2q3), L2p = zbuf(ctx, 9, c2q3);
-  if (!L2p.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-  {
-    // de-interleave: permute [n | 2] -> [2 | n]
-    HS_TRY(ctx->r[2].ensure(2 * cqc * 8));
-    HS_TRY(permute(ctx, dense({c2, 2}), dense({2, c2}), {1, 0}, ctx->r[0].d(), ctx->r[2].d()));
-    HS_CUDA(cudaMemcpyAsync(Cz.re, ctx->r[2].d(), c2 * 8, cudaMemcpyDeviceToDevice, s));
-    HS_CUDA(cudaMemcpyAsync(Cz.im, ctx->r[2].d() + c2, c2 * 8, cudaMemcpyDeviceToDevice, s));
-    HS_TRY(permute(ctx, dense({cqc, 2}), dense({2, cqc}), {1, 0}, ctx->r[1].d(), ctx->r[2].d()));
-    HS_CUDA(cudaMemcpyAsync(Tz.re, ctx->r[2].d(), cqc * 8, cudaMemcpyDeviceToDevice, s));
-    HS_CUDA(cudaMemcpyAsync(Tz.im, ctx->r[2].d() + cqc, cqc * 8, cudaMemcpyDeviceToDevice, s));
-  }
-  HS_TRY(zpermute(ctx, dense({chi, chi}), dense({chi, chi}), {1, 0}, Cz, Ctz));                 // C^T
-  HS_TRY(zpermute(ctx, dense({chi, q, chi}), dense({q, chi, chi}), {1, 2, 0}, Tz, Tqz));       // Tq[(x,e)|c]
-  HS_TRY(zgemm(ctx, dense_gemm(chi, q * chi, chi), Cz, Tqz, H1));                               // H1[a|(x,e)]
-  HS_TRY(zgemm(ctx, dense_gemm(chi * q, chi, chi), H1, Ctz, Hz));                               // H[(a,x)|b]
-  HS_TRY(zpermute(ctx, dense({chi, q, chi}), dense({q, chi, chi}), {1, 2, 0}, Hz, Hq));        // Hq[(l,e)|c]
-  if (kind == HS_RDM_ENV_ONE_SITE) {
-    // eps[u,l,d,r] = H[a,u,b] T[b,r,b'] H[b',d,a'] T[a',l,a] (the clockwise ring of Eq. (4))
-    ZBuf Y1 = zbuf(ctx, 7, c2q2), Y2 = zbuf(ctx, 8, c2q3), Y2p = zbuf(ctx, 9, c2q3), Tl = zbuf(ctx, 10, cqc),
-         E3 = zbuf(ctx, 11, q * q * q * q);
-    if (!E3.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-    HS_TRY(zgemm(ctx, dense_gemm(chi * q, q * chi, chi), Hz, Tqz, Y1));                        // [(a,u)|(r,b')]
-    HS_TRY(zgemm(ctx, dense_gemm(chi * q * q, q * chi, chi), Y1, Hq, Y2));                     // [(a,u,r)|(d,a')]
-    HS_TRY(zpermute(ctx, dense({chi, q, q, q, chi}), dense({q, q, q, chi, chi}), {1, 2, 3, 4, 0}, Y2, Y2p));
-    HS_TRY(zpermute(ctx, dense({chi, q, chi}), dense({q, chi, chi}), {1, 0, 2}, Tz, Tl));      // Tl[l|(a',a)]
-    HS_TRY(zgemm(ctx, dense_gemm(q * q * q, q, chi * chi), Y2p, Tl, E3));                       // [(u,r,d)|l]
-    // eps[u,l,d,r] (interleaved complex): permute each part, then interleave
-    ZBuf Eo = zbuf(ctx, 12, q * q * q * q);
-    if (!Eo.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-    HS_TRY(zpermute(ctx, dense({q, q, q, q}), dense({q, q, q, q}), {0, 3, 2, 1}, E3, Eo));
-    const long long n4 = q * q * q * q;
-    HS_TRY(ctx->r[2].ensure(2 * n4 * 8));
-    HS_CUDA(cudaMemcpyAsync(ctx->r[2].d(), Eo.re, n4 * 8, cudaMemcpyDeviceToDevice, s));
-    HS_CUDA(cudaMemcpyAsync(ctx->r[2].d() + n4, Eo.im, n4 * 8, cudaMemcpyDeviceToDevice, s));
-    return permute(ctx, dense({2, n4}), dense({n4, 2}), {1, 0}, ctx->r[2].d(), out);
-  }
-  HS_TRY(zgemm(ctx, dense_gemm(chi * q, q * chi, chi), Tz, Hq, L1));                            // L1[(b,d1)|(l1,e)]
-  HS_TRY(zgemm(ctx, dense_gemm(chi * q * q, q * chi, chi), L1, Tqz, L2));                       // L2[(b,d1,l1)|(u1,t)]
-  HS_TRY(zpermute(ctx, dense({chi, q, q, q, chi}), dense({chi, chi, q, q, q}), {0, 4, 1, 2, 3}, L2, L2p));
-  // open double layers: a1[(s,s',r) | (d,l,u)], a2[(s,s',l) | (u,r,d)]
-  const long long nao = d2 * q * q * q * q;
-  ZBuf a1 = zbuf(ctx, 10, nao), a2 = zbuf(ctx, 11, nao);
-  if (!a2.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-  hs_launch(open_double_layer_c_kernel, grid_for(nao), 256, 0, s, A, d, D, make_int4(3, 2, 1, 0), a1.re, a1.im);
-  HS_CUDA(cudaGetLastError());
-  hs_launch(open_double_layer_c_kernel, grid_for(nao), 256, 0, s, A, d, D, make_int4(1, 0, 3, 2), a2.re, a2.im);
-  HS_CUDA(cudaGetLastError());
-  ctx->launches += 2;
-  ZBuf LB = zbuf(ctx, 1, c2 * d2 * q), RB = zbuf(ctx, 2, c2 * d2 * q);  // reuse (T, C^T no longer needed)
-  ZBuf LBp = zbuf(ctx, 4, c2 * d2 * q), RBp = zbuf(ctx, 5, c2 * d2 * q), R4 = zbuf(ctx, 0, d2 * d2);
-  if (!R4.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-  HS_TRY(zgemm(ctx, dense_gemm(c2, d2 * q, q * q * q), L2p, a1, LB));                           // LB[(b,t)|(s,s',m)]
-  HS_TRY(zgemm(ctx, dense_gemm(c2, d2 * q, q * q * q), L2p, a2, RB));                           // RB[(t,b)|(s,s',m)]
-  HS_TRY(zpermute(ctx, dense({chi, chi, d, d, q}), dense({d, d, chi, chi, q}), {2, 3, 0, 1, 4}, LB, LBp));
-  HS_TRY(zpermute(ctx, dense({chi, chi, d, d, q}), dense({d, d, chi, chi, q}), {2, 3, 1, 0, 4}, RB, RBp));
-  HS_TRY(zgemm(ctx, dense_gemm(d2, d2, c2 * q), LBp, RBp, R4));                                 // rho4
-  hs_launch(finish_rho_c_kernel, 1, 256, 0, s, R4.re, R4.im, d, h, out, tr_out);
-  HS_CUDA(cudaGetLastError());
-  ctx->launches += 1;
-  return HS_OK;
-}
-
-// Adjoint of rdm_complex with the environment fixed: drho (interleaved
-// complex d^4, cotangent dE/dRe rho + i dE/dIm rho) -> dA (interleaved complex).
-hs_status rdm_vjp_complex(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, const double* drho,
-                          double* dA_out) {
-  cudaStream_t s = ctx->stream;
-  const long long chi = env->chi_even + env->chi_odd, q = (long long)D * D, d2 = (long long)d * d;
-  const long long c2 = chi * chi, c2q3 = c2 * q * q * q, nb = c2 * d2 * q;
-  // forward: leaves L2p (slot 9), LB (1), RB (2), LBp (4), RBp (5)
-  HS_TRY(ctx->r[3].ensure(2 * d2 * d2 * 8 + 4 * 8));
-  HS_TRY(rdm_complex(ctx, env, A, d, D, HS_RDM_TWO_SITE, nullptr, ctx->r[3].d(), ctx->r[3].d() + 2 * d2 * d2));
-  ZBuf L2p = zbuf(ctx, 9, c2q3), LBp = zbuf(ctx, 4, nb), RBp = zbuf(ctx, 5, nb);
-  // cotangent of rho4[s1, s1', s2, s2'] and of its transpose
-  ZBuf G = zbuf(ctx, 12, d2 * d2), G4 = zbuf(ctx, 13, d2 * d2), G4t = zbuf(ctx, 14, d2 * d2);
-  if (!G4t.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-  HS_TRY(ctx->r[4].ensure(2 * d2 * d2 * 8));
-  HS_TRY(permute(ctx, dense({d2 * d2, 2}), dense({2, d2 * d2}), {1, 0}, drho, ctx->r[4].d()));
-  HS_CUDA(cudaMemcpyAsync(G.re, ctx->r[4].d(), d2 * d2 * 8, cudaMemcpyDeviceToDevice, s));
-  HS_CUDA(cudaMemcpyAsync(G.im, ctx->r[4].d() + d2 * d2, d2 * d2 * 8, cudaMemcpyDeviceToDevice, s));
-  HS_TRY(zpermute(ctx, dense({d, d, d, d}), dense({d, d, d, d}), {0, 2, 1, 3}, G, G4));
-  HS_TRY(zpermute(ctx, dense({d2, d2}), dense({d2, d2}), {1, 0}, G4, G4t));
-  // gLBp = G4 conj(RBp), gRBp = G4^T conj(LBp): B operands transposed to [(b,t,m) | (s,s')]
-  ZBuf RBq = zbuf(ctx, 15, nb), LBq = zbuf(ctx, 16, nb), gLBp = zbuf(ctx, 17, nb), gRBp = zbuf(ctx, 18, nb);
-  if (!gRBp.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-  HS_TRY(zpermute(ctx, dense({d2, c2 * q}), dense({c2 * q, d2}), {1, 0}, RBp, RBq));
-  HS_TRY(zpermute(ctx, dense({d2, c2 * q}), dense({c2 * q, d2}), {1, 0}, LBp, LBq));
-  HS_TRY(zgemm(ctx, dense_gemm(d2, c2 * q, d2), G4, RBq, gLBp, true));
-  HS_TRY(zgemm(ctx, dense_gemm(d2, c2 * q, d2), G4t, LBq, gRBp, true));
-  // back to [(s, s', m) | (b, t)] and [(s, s', m) | (t, b)] (LB rows (b,t), RB rows (t,b))
-  ZBuf gLm = zbuf(ctx, 15, nb), gRm = zbuf(ctx, 16, nb);
-  HS_TRY(zpermute(ctx, dense({d, d, chi, chi, q}), dense({d, d, q, chi, chi}), {0, 1, 4, 2, 3}, gLBp, gLm));
-  HS_TRY(zpermute(ctx, dense({d, d, chi, chi, q}), dense({d, d, q, chi, chi}), {0, 1, 4, 3, 2}, gRBp, gRm));
-  // open double layers: g_a = g_B^T conj(L2p) with L2p^T[(k0,k1,k2) | (x0, x4)]
-  ZBuf L2pT = zbuf(ctx, 8, c2q3);
-  if (!L2pT.re) return fail(HS_ERR_CUDA, "workspace allocation failed");
-  HS_TRY(zpermute(ctx, dense({c2, q * q * q}), dense({q * q * q, c2}), {1, 0}, L2p, L2pT));
-  const long long nao = d2 * q * q * q * q;
-  ZBuf g1 = zbuf(ctx, 10, nao), g2 = zbuf(ctx, 11, nao);
-  HS_TRY(zgemm(ctx, dense_gemm(d2 * q, q * q * q, c2), gLm, L2pT, g1, true));
-  HS_TRY(zgemm(ctx, dense_gemm(d2 * q, q * q * q, c2), gRm, L2pT, g2, true));
-  const long long nA = (long long)d * D * D * D * D;
-  hs_launch(open_double_layer_c_vjp_kernel, grid_for(nA), 256, 0, s, g1.re, g1.im, make_int4(3, 2, 1, 0), g2.re, g2.im,
-                                                               make_int4(1, 0, 3, 2), A, d, D, dA_out);
-  HS_CUDA(cudaGetLastError());
-  ctx->launches += 1;
-  return HS_OK;
-}
-
-// Shared forward chain of the two-site network up to the half-network blocks:
-// on return r[8] = Z2 [(l,u,t')|(d,b')], r[9] = Z2p [(t',b')|(l,u,d)],
-// r[10]/r[11] = open double layers of the left/right site, r[12]/r[13] =
-// LB/RB [(t',b')|(s,s',m)], r[14]/r[15] = LBp/RBp [(s,s')|(t',b',m)],
-// r[6] = rho4 [(s1,s1')|(s2,s2')]. kind selects how far it goes.
-hs_status rdm_chain(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, hs_rdm_kind kind,
-                    double* eps_out) {
-  cudaStream_t s = ctx->stream;
-  const hs_gemm_backend be = env->gemm_backend;
-  const long long chi = env->chi_even + env->chi_odd, q = (long long)D * D;
-  const long long c2 = chi * chi, cqc = chi * q * chi, c2q2 = c2 * q * q, c2q3 = c2q2 * q;
-  DBuf* r = ctx->r;
-  HS_TRY(r[0].ensure(c2 * 8));
-  HS_TRY(r[1].ensure(cqc * 8));
-  HS_TRY(r[2].ensure(cqc * 8));
-  HS_TRY(r[3].ensure(cqc * 8));
-  HS_TRY(r[4].ensure(cqc * 8));
-  HS_TRY(r[5].ensure(cqc * 8));
-  HS_TRY(r[6].ensure((c2q2 > c2 ? c2q2 : c2) * 8));
-  HS_TRY(r[7].ensure(c2q2 * 8));
-  HS_TRY(r[8].ensure(c2q3 * 8));
-  HS_TRY(r[9].ensure(c2q3 * 8));
-  double *Cd = r[0].d(), *Td = r[1].d(), *Tsw = r[2].d(), *E1 = r[3].d(), *E = r[4].d(),
-         *Ep = r[5].d(), *Z1 = r[6].d(), *Z1p = r[7].d(), *Z2 = r[8].d(), *Z2p = r[9].d();
-
-  // environment in the plain combined basis
-  HS_CUDA(launch_env_to_dense(env->C, env->T, D, env->chi_even, env->chi_odd,
-                              env->basis == HS_BASIS_HERMITIAN, Cd, Td, s));
-  // Tsw[(x, b) | a] = T[a, x, b]
-  HS_TRY(permute(ctx, dense({chi, q, chi}), dense({q, chi, chi}), {1, 2, 0}, Td, Tsw));
-  // half ring E[t, l, b] = C[t, a] T[a, l, a'] C[a', b]
-  HS_TRY(gemm(ctx, be, dense_gemm(chi, q * chi, chi), Cd, Tsw, E1));          // E1[t | (l, a')]
-  HS_TRY(permute(ctx, dense({chi, chi}), dense({chi, chi}), {1, 0}, Cd, Z1));  // C^T in Z1
-  HS_TRY(gemm(ctx, be, dense_gemm(chi * q, chi, chi), E1, Z1, E));             // E[(t, l) | b]
-  // Z1[l, b, u, t'] = E[t, l, b] T[t, u, t']
-  HS_TRY(permute(ctx, dense({chi, q, chi}), dense({q, chi, chi}), {1, 2, 0}, E, Ep));   // Ep[(l,b)|t]
-  HS_TRY(gemm(ctx, be, dense_gemm(q * chi, q * chi, chi), Ep, Tsw, Z1));
-  // Z2[l, u, t', d, b'] = Z1[l, b, u, t'] T[b, d, b']
-  HS_TRY(permute(ctx, dense({q, chi, q, chi}), dense({q, q, chi, chi}), {0, 2, 3, 1}, Z1, Z1p));
-  HS_TRY(gemm(ctx, be, dense_gemm(q * q * chi, q * chi, chi), Z1p, Tsw, Z2));
-
-  if (kind == HS_RDM_ENV_ONE_SITE) {
-    // Z2 plays Y2[u, l, a', r, b']; eps[u,l,r,d] = Y2[u,l,a',r,b'] H[a',d,b'], H = E
-    HS_TRY(r[12].ensure(cqc * 8));
-    HS_TRY(r[13].ensure(q * q * q * q * 8));
-    HS_TRY(permute(ctx, dense({q * q, chi, q, chi}), dense({q * q, q, chi, chi}), {0, 2, 1, 3}, Z2, Z2p));
-    HS_TRY(permute(ctx, dense({chi, q, chi}), dense({q, chi, chi}), {1, 0, 2}, E, r[12].d()));  // Hd[d|(a',b')]
-    HS_TRY(gemm(ctx, be, dense_gemm(q * q * q, q, chi * chi), Z2p, r[12].d(), r[13].d()));     // [(u,l,r)|d]
-    HS_TRY(permute(ctx, dense({q * q, q, q}), dense({q * q, q, q}), {0, 2, 1}, r[13].d(), eps_out));
-    return HS_OK;
-  }
-
-  const long long d2 = (long long)d * d;
-  HS_TRY(r[10].ensure(d2 * q * q * q * q * 8));
-  HS_TRY(r[11].ensure(d2 * q * q * q * q * 8));
-  HS_TRY(r[12].ensure(c2 * d2 * q * 8));
-  HS_TRY(r[13].ensure(c2 * d2 * q * 8));
-  HS_TRY(r[14].ensure(c2 * d2 * q * 8));
-  HS_TRY(r[15].ensure(c2 * d2 * q * 8));
-  double *aoL = r[10].d(), *aoR = r[11].d(), *LB = r[12].d(), *RB = r[13].d(), *LBp = r[14].d(),
-         *RBp = r[15].d();
-  const long long nao = d2 * q * q * q * q;
-  hs_launch(open_double_layer_kernel, grid_for(nao), 256, 0, s, A, d, D, true, aoL);
-  HS_CUDA(cudaGetLastError());
-  hs_launch(open_double_layer_kernel, grid_for(nao), 256, 0, s, A, d, D, false, aoR);
-  HS_CUDA(cudaGetLastError());
-  // Z2p[(t', b') | (l, u, d)]
-  HS_TRY(permute(ctx, dense({q * q, chi, q, chi}), dense({chi, chi, q * q, q}), {1, 3, 0, 2}, Z2, Z2p));
-  // LB[(t', b') | (s, s', m)] over (l, u, d); RB over (r, u, d) of the mirror site
-  HS_TRY(gemm(ctx, be, dense_gemm(c2, d2 * q, q * q * q), Z2p, aoL, LB));
-  HS_TRY(gemm(ctx, be, dense_gemm(c2, d2 * q, q * q * q), Z2p, aoR, RB));
-  // [(s, s') | (t', b', m)]
-  HS_TRY(permute(ctx, dense({c2, d2, q}), dense({d2, c2, q}), {1, 0, 2}, LB, LBp));
-  HS_TRY(permute(ctx, dense({c2, d2, q}), dense({d2, c2, q}), {1, 0, 2}, RB, RBp));
-  HS_TRY(gemm(ctx, be, dense_gemm(d2, d2, c2 * q), LBp, RBp, Z1));  // rho4[(s1,s1') | (s2,s2')]
-  return HS_OK;
-}
-
-static hs_status rdm_vjp_after_chain(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, const double* drho,
-                                     double* dA_out);
 
 namespace hs {
 // The open double layers of the two-site network (left site open on r, right
@@ -665,10 +806,7 @@ extern "C" hs_status hs_rdm(hs_ctx ctx, const hs_env* env, const double* A, int 
     const long long q = (long long)D * D, n4 = q * q * q * q;
     DBuf& eps = ctx->hb[11];
     HS_TRY(eps.ensure((size_t)n4 * (cplx ? 2 : 1) * sizeof(double)));
-    if (cplx)
-      HS_TRY(rdm_complex(ctx, env, A, d, D, HS_RDM_ENV_ONE_SITE, nullptr, eps.d(), nullptr));
-    else
-      HS_TRY(rdm_chain(ctx, env, A, d, D, HS_RDM_ENV_ONE_SITE, eps.d()));
+    HS_TRY(one_site_chain(ctx, env, d, D, eps.d()));
     hs_launch(one_site_rho_kernel, d * d, 256, 0, ctx->stream, eps.d(), A, d, D, cplx, out);
     HS_CUDA(cudaGetLastError());
     hs_launch(finish_rho1_kernel, 1, 32, 0, ctx->stream, out, d, cplx, h, tr_out);
@@ -676,13 +814,9 @@ extern "C" hs_status hs_rdm(hs_ctx ctx, const hs_env* env, const double* A, int 
     ctx->launches += 2;
     return HS_OK;
   }
-  if (dtype == HS_C128) return rdm_complex(ctx, env, A, d, D, kind, h, out, tr_out);
-  HS_TRY(rdm_chain(ctx, env, A, d, D, kind, out));
-  if (kind == HS_RDM_ENV_ONE_SITE) return HS_OK;
-  hs_launch(finish_rho_kernel, 1, 256, 0, ctx->stream, ctx->r[6].d(), d, env->basis == HS_BASIS_HERMITIAN, h, out,
-                                                tr_out);
-  HS_CUDA(cudaGetLastError());
-  return HS_OK;
+  if (kind == HS_RDM_ENV_ONE_SITE) return one_site_chain(ctx, env, d, D, out);
+  HS_TRY(rdm_chain(ctx, env, A, d, D));
+  return finish_rdm(ctx, env, d, D, h, out, tr_out);
 }
 
 extern "C" hs_status hs_rdm_vjp(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, hs_dtype dtype,
@@ -691,9 +825,8 @@ extern "C" hs_status hs_rdm_vjp(hs_ctx ctx, const hs_env* env, const double* A, 
   if (!env || !A || !drho || !dA_out || d <= 0 || D != env->D) return fail(HS_ERR_INVALID_ARG, "bad arguments");
   if (dtype != HS_F64 && dtype != HS_C128) return fail(HS_ERR_DTYPE, "unknown dtype");
   if ((dtype == HS_C128) != (env->dtype == HS_C128)) return fail(HS_ERR_DTYPE, "A and environment disagree on dtype");
-  if (dtype == HS_C128) return rdm_vjp_complex(ctx, env, A, d, D, drho, dA_out);
-  HS_TRY(rdm_chain(ctx, env, A, d, D, HS_RDM_TWO_SITE, nullptr));
-  return rdm_vjp_after_chain(ctx, env, A, d, D, drho, dA_out);
+  HS_TRY(rdm_chain(ctx, env, A, d, D));
+  return rdm_vjp_after_chain(ctx, env, d, D, A, drho, dA_out);
 }
 
 extern "C" hs_status hs_energy_vjp(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, hs_dtype dtype,
@@ -710,64 +843,11 @@ extern "C" hs_status hs_energy_vjp(hs_ctx ctx, const hs_env* env, const double* 
   double* rho = w.d();
   double* drho = rho + (long long)n * n * (cplx ? 2 : 1);
   double* tr = drho + (long long)n * n * (cplx ? 2 : 1);
-  if (cplx) {
-    HS_TRY(rdm_complex(ctx, env, A, d, D, HS_RDM_TWO_SITE, h, rho, tr));
-  } else {
-    HS_TRY(rdm_chain(ctx, env, A, d, D, HS_RDM_TWO_SITE, nullptr));
-    hs_launch(finish_rho_kernel, 1, 256, 0, ctx->stream, ctx->r[6].d(), d, env->basis == HS_BASIS_HERMITIAN, h, rho,
-              tr);
-    HS_CUDA(cudaGetLastError());
-  }
+  HS_TRY(rdm_chain(ctx, env, A, d, D));
+  HS_TRY(finish_rdm(ctx, env, d, D, h, rho, tr));
   hs_launch(energy_cotangent_kernel, 1, 256, 0, ctx->stream, (const double*)tr, h, n, cplx, dE, drho);
   HS_CUDA(cudaGetLastError());
-  ctx->launches += 2;
-  if (cplx) return rdm_vjp_complex(ctx, env, A, d, D, drho, dA_out);
-  return rdm_vjp_after_chain(ctx, env, A, d, D, drho, dA_out);
+  ctx->launches += 1;
+  return rdm_vjp_after_chain(ctx, env, d, D, A, drho, dA_out);
 }
 
-// Reverse pass of the real two-site chain; rdm_chain(HS_RDM_TWO_SITE) must have
-// run on the same environment and A just before (its buffers r[8..15]).
-static hs_status rdm_vjp_after_chain(hs_ctx ctx, const hs_env* env, const double* A, int d, int D, const double* drho,
-                                     double* dA_out) {
-  cudaStream_t s = ctx->stream;
-  const hs_gemm_backend be = env->gemm_backend;
-  const long long chi = env->chi_even + env->chi_odd, q = (long long)D * D, c2 = chi * chi,
-                  d2 = (long long)d * d;
-  DBuf* r = ctx->r;
-  double *Z2 = r[8].d(), *Z2p = r[9].d(), *LB = r[12].d(), *RB = r[13].d();
-  // rho[(s1 s2), (s1' s2')] = rho4[s1, s1', s2, s2']: cotangent of rho4 and its transpose
-  HS_TRY(ctx->hb[0].ensure(2 * d2 * d2 * 8));
-  double* drho4 = ctx->hb[0].d();
-  double* drho4T = drho4 + d2 * d2;
-  HS_TRY(permute(ctx, dense({d, d, d, d}), dense({d, d, d, d}), {0, 2, 1, 3}, drho, drho4));
-  HS_TRY(permute(ctx, dense({d2, d2}), dense({d2, d2}), {1, 0}, drho4, drho4T));
-  // RBq/LBq[(t', b', m) | (s, s')]
-  HS_TRY(ctx->hb[1].ensure(c2 * d2 * q * 8));
-  HS_TRY(ctx->hb[2].ensure(c2 * d2 * q * 8));
-  HS_TRY(ctx->hb[3].ensure(c2 * d2 * q * 8));
-  HS_TRY(ctx->hb[4].ensure(c2 * d2 * q * 8));
-  double *LBq = ctx->hb[1].d(), *RBq = ctx->hb[2].d(), *dLB = ctx->hb[3].d(), *dRB = ctx->hb[4].d();
-  HS_TRY(permute(ctx, dense({c2, d2, q}), dense({c2, q, d2}), {0, 2, 1}, LB, LBq));
-  HS_TRY(permute(ctx, dense({c2, d2, q}), dense({c2, q, d2}), {0, 2, 1}, RB, RBq));
-  // dLB[(s1,s1') | (t',b',m)] = drho4 RB ; dRB[(s2,s2') | (t',b',m)] = drho4^T LB
-  HS_TRY(gemm(ctx, be, dense_gemm(d2, c2 * q, d2), drho4, RBq, dLB));
-  HS_TRY(gemm(ctx, be, dense_gemm(d2, c2 * q, d2), drho4T, LBq, dRB));
-  // [(s, s', m) | (t', b')]
-  HS_TRY(ctx->hb[5].ensure(c2 * d2 * q * 8));
-  HS_TRY(ctx->hb[6].ensure(c2 * d2 * q * 8));
-  double *dLBm = ctx->hb[5].d(), *dRBm = ctx->hb[6].d();
-  HS_TRY(permute(ctx, dense({d2, c2, q}), dense({d2, q, c2}), {0, 2, 1}, dLB, dLBm));
-  HS_TRY(permute(ctx, dense({d2, c2, q}), dense({d2, q, c2}), {0, 2, 1}, dRB, dRBm));
-  // Z2t[(l, u, d) | (t', b')] from Z2[(l,u), t', d, b']
-  HS_TRY(permute(ctx, dense({q * q, chi, q, chi}), dense({q * q, q, chi, chi}), {0, 2, 1, 3}, Z2, Z2p));
-  // cotangents of the open double layers: dao[(s, s', m) | (c0, u, d)]
-  const long long nao = d2 * q * q * q * q;
-  HS_TRY(ctx->hb[7].ensure(nao * 8));
-  HS_TRY(ctx->hb[8].ensure(nao * 8));
-  HS_TRY(gemm(ctx, be, dense_gemm(d2 * q, q * q * q, c2), dLBm, Z2p, ctx->hb[7].d()));
-  HS_TRY(gemm(ctx, be, dense_gemm(d2 * q, q * q * q, c2), dRBm, Z2p, ctx->hb[8].d()));
-  const long long nA = (long long)d * D * D * D * D;
-  hs_launch(open_double_layer_vjp_kernel, grid_for(nA), 256, 0, s, ctx->hb[7].d(), ctx->hb[8].d(), A, d, D, dA_out);
-  HS_CUDA(cudaGetLastError());
-  return HS_OK;
-}
