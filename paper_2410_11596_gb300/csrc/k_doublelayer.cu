@@ -156,67 +156,142 @@ __global__ void double_layer_graded_kernel(const double* __restrict__ A, int d, 
   }
 }
 
-__global__ void double_layer_dense_kernel(const double* __restrict__ A, int d, int D, bool cplx,
-                                          double* __restrict__ out) {
+// One warp per row (x_u, x_l, x_d) of q contiguous entries: the row's ket and
+// bra offsets into A once, 32-bit indices inside. Bound by the FP64 pipe (d FMAs
+// per entry) and the write.
+__global__ void __launch_bounds__(256) double_layer_dense_kernel(const double* __restrict__ A, int d, int D, bool cplx,
+                                                                 double* __restrict__ out) {
   hs_pdl_enter();
-  const int q = D * D;
-  const long long total = (long long)q * q * q * q;
-  const long long D4 = (long long)D * D * D * D;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int xr = (int)(e % q), xd = (int)((e / q) % q), xl = (int)((e / q / q) % q),
-              xu = (int)(e / q / q / q);
-    const long long ik = (((long long)(xu % D) * D + xl % D) * D + xd % D) * D + xr % D;
-    const long long ib = (((long long)(xu / D) * D + xl / D) * D + xd / D) * D + xr / D;
-    if (!cplx) {
-      double s = 0.0;
-      for (int p = 0; p < d; ++p) s += A[p * D4 + ik] * A[p * D4 + ib];
-      out[e] = s;
-    } else {
-      double re = 0.0, im = 0.0;
-      for (int p = 0; p < d; ++p) {
-        const double ar = A[2 * (p * D4 + ik)], ai = A[2 * (p * D4 + ik) + 1];
-        const double br = A[2 * (p * D4 + ib)], bi = -A[2 * (p * D4 + ib) + 1];
-        re += ar * br - ai * bi;
-        im += ar * bi + ai * br;
+  extern __shared__ int2 halves[];  // x -> (ket, bra)
+  const int q = D * D, lane = threadIdx.x % 32;
+  for (int x = threadIdx.x; x < q; x += blockDim.x) halves[x] = make_int2(x % D, x / D);
+  __syncthreads();
+  const long long rows = (long long)q * q * q;
+  const int D4 = D * D * D * D;
+  for (long long r = (long long)blockIdx.x * 8 + threadIdx.x / 32; r < rows; r += (long long)gridDim.x * 8) {
+    const int xd = (int)(r % q), xl = (int)(r / q % q), xu = (int)(r / q / q);
+    const int2 hu = halves[xu], hl = halves[xl], hd = halves[xd];
+    const int kr = ((hu.x * D + hl.x) * D + hd.x) * D, br = ((hu.y * D + hl.y) * D + hd.y) * D;
+    double* o = out + (cplx ? 2 : 1) * r * q;
+    for (int x = lane; x < q; x += 32) {
+      const int ik = kr + halves[x].x, ib = br + halves[x].y;
+      if (!cplx) {
+        double s = 0.0;
+        for (int p = 0; p < d; ++p) s += A[(long long)p * D4 + ik] * A[(long long)p * D4 + ib];
+        o[x] = s;
+      } else {
+        double re = 0.0, im = 0.0;
+        for (int p = 0; p < d; ++p) {
+          const double ar = A[2 * ((long long)p * D4 + ik)], ai = A[2 * ((long long)p * D4 + ik) + 1];
+          const double br_ = A[2 * ((long long)p * D4 + ib)], bi = -A[2 * ((long long)p * D4 + ib) + 1];
+          re += ar * br_ - ai * bi;
+          im += ar * bi + ai * br_;
+        }
+        o[2 * x] = re;
+        o[2 * x + 1] = im;
       }
-      out[2 * e] = re;
-      out[2 * e + 1] = im;
     }
   }
 }
 
-__global__ void rotate_dense_kernel(const double* __restrict__ a, int D, double* __restrict__ out,
-                                    unsigned long long* maxes) {
+// Rotation of a dense double layer into the eigenbasis of S. On one leg a basis
+// pair (k < l) turns the plain states (k l') and (l k') into an even and an odd
+// state, a sum and a difference; so the 16 plain entries of four such pairs give
+// the 16 rotated ones by four rounds of sums and differences. One thread per
+// four leg classes P (P < D: the state (P P'), else pair P - D): every plain
+// entry is read once, 4 additions an entry (16 gathered reads and 16 FMAs of a
+// product of four coefficients before: 1354 us at D = 7, now bound by the FP64
+// pipe). Lanes run over the last leg, whose row of q entries they share.
+__global__ void __launch_bounds__(256) rotate_dense_kernel(const double* __restrict__ a, int D, double* __restrict__ out,
+                                                           unsigned long long* maxes) {
   hs_pdl_enter();
-  const int q = D * D;
-  const int qe = D * (D + 1) / 2, qo = q - qe;
-  const long long total = (long long)q * q * q * q;
-  double mall = 0.0, modd = 0.0;
+  extern __shared__ int2 pairs[];  // class -> (x of (k l'), x of (l k')), equal for a diagonal class
+  const int q = D * D, ne = D * (D + 1) / 2, no = q - ne;
+  for (int P = threadIdx.x; P < ne; P += blockDim.x) {
+    int k = P, l = P;
+    if (P >= D) pair_of(P - D, D, &k, &l);
+    pairs[P] = make_int2(k + D * l, l + D * k);
+  }
+  __syncthreads();
+  const long long total = (long long)ne * ne * ne * ne;
+  const long long rows0 = (long long)ne * ne + (long long)no * no, rows1 = 2LL * ne * no;
+  constexpr unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
+  unsigned long long mall = 0, modd = 0;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
-    const int Xr = (int)(e % q), Xd = (int)((e / q) % q), Xl = (int)((e / q / q) % q),
-              Xu = (int)(e / q / q / q);
-    const Terms tu = basis_terms(Xu, D, true), tl = basis_terms(Xl, D, true),
-                td = basis_terms(Xd, D, true), tr = basis_terms(Xr, D, true);
-    double acc = 0.0;
-    for (int i = 0; i < tu.n; ++i)
-      for (int j = 0; j < tl.n; ++j)
-        for (int k = 0; k < td.n; ++k)
-          for (int m = 0; m < tr.n; ++m) {
-            const long long x = (((long long)(tu.ket[i] + D * tu.bra[i]) * q + (tl.ket[j] + D * tl.bra[j])) * q +
-                                 (td.ket[k] + D * td.bra[k])) * q + (tr.ket[m] + D * tr.bra[m]);
-            acc += tu.c[i] * tl.c[j] * td.c[k] * tr.c[m] * a[x];
-          }
-    const long long pos = fso4(Xu, Xl, Xd, Xr, qe, qo);
-    mall = fmax(mall, fabs(acc));
-    if (pos < 0)
-      modd = fmax(modd, fabs(acc));
-    else
-      out[pos] = acc;
+    int P[4];
+    // (ne^2)^2 classes: one 64-bit division, the rest in 32 bits
+    const unsigned hi = (unsigned)(e / (ne * ne)), lo = (unsigned)(e - (long long)hi * (ne * ne));
+    P[0] = (int)(hi / ne);
+    P[1] = (int)(hi % ne);
+    P[2] = (int)(lo / ne);
+    P[3] = (int)(lo % ne);
+    int2 x[4];
+    int off = 0;  // legs with two states, as a mask (bit 3: the first leg)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      x[j] = pairs[P[j]];
+      if (P[j] >= D) off |= 8 >> j;
+    }
+    // scale = 2^(-n / 2) for n two-state legs, each power rounded once
+    const int n = __popc(off);
+    const double scale = n == 0 ? 1.0 : n == 1 ? 0.70710678118654752440 : n == 2 ? 0.5 : n == 3 ? 0.35355339059327376220 : 0.25;
+    double v[16];
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      v[m] = 0.0;
+      if ((m & ~off) == 0) {
+        const long long xu = m & 8 ? x[0].y : x[0].x, xl = m & 4 ? x[1].y : x[1].x;
+        const int xd = m & 2 ? x[2].y : x[2].x, xr = m & 1 ? x[3].y : x[3].x;
+        v[m] = a[((xu * q + xl) * q + xd) * q + xr];
+      }
+    }
+#pragma unroll
+    for (int b = 1; b < 16; b <<= 1) {
+      if (!(off & b)) continue;
+#pragma unroll
+      for (int m = 0; m < 16; ++m)
+        if (!(m & b)) {
+          const double p = v[m], w = v[m | b];
+          v[m] = p + w;
+          v[m | b] = p - w;
+        }
+    }
+    unsigned long long odd = 0;  // largest odd-total entry before the scale
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      if ((m & ~off) != 0) continue;
+      const int pu = m >> 3 & 1, pl = m >> 2 & 1, pd = m >> 1 & 1, pr = m & 1;
+      const bool is_odd = (pu + pl + pd + pr) & 1;
+      const double w = is_odd ? v[m] : scale * v[m];
+      unsigned long long mag = (unsigned long long)__double_as_longlong(w) & kMag;
+      if (mag > 0x7FF0000000000000ull) mag = 0;  // a NaN does not count
+      if (is_odd) {
+        odd = odd > mag ? odd : mag;
+        continue;
+      }
+      mall = mall > mag ? mall : mag;
+      // FSO position: block pu ^ pl, tuples (0 0), (1 1) or (0 1), (1 0)
+      const int blk = pu ^ pl;
+      const long long iu = P[0] - pu * D, il = P[1] - pl * D, id = P[2] - pd * D, ir = P[3] - pr * D;
+      const long long tr = pu ? (blk ? (long long)ne * no : (long long)ne * ne) : 0;
+      const long long tc = pd ? (blk ? (long long)ne * no : (long long)ne * ne) : 0;
+      const long long row = tr + iu * (pl ? no : ne) + il, col = tc + id * (pr ? no : ne) + ir;
+      out[blk ? rows0 * rows0 + row * rows1 + col : row * rows0 + col] = w;
+    }
+    odd = (unsigned long long)__double_as_longlong(scale * __longlong_as_double((long long)odd));
+    modd = modd > odd ? modd : odd;
+    mall = mall > odd ? mall : odd;
   }
-  atomicMax(&maxes[0], (unsigned long long)__double_as_longlong(modd));
-  atomicMax(&maxes[1], (unsigned long long)__double_as_longlong(mall));
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long x = __shfl_xor_sync(0xffffffffu, mall, o), y = __shfl_xor_sync(0xffffffffu, modd, o);
+    mall = mall > x ? mall : x;
+    modd = modd > y ? modd : y;
+  }
+  if (threadIdx.x % 32 == 0) {
+    atomicMax(&maxes[0], modd);
+    atomicMax(&maxes[1], mall);
+  }
 }
 
 // Index of the Hermitian basis state pair (k, l), k < l, lexicographic (the
@@ -320,7 +395,9 @@ cudaError_t launch_double_layer_graded(const double* A, int d, int D, double* ou
 cudaError_t launch_double_layer_dense(const double* A, int d, int D, bool cplx, double* out,
                                       cudaStream_t s) {
   const long long q = (long long)D * D;
-  hs_launch(double_layer_dense_kernel, grid_for(q * q * q * q), 256, 0, s, A, d, D, cplx, out);
+  long long g = (q * q * q + 7) / 8;
+  if (g > 16LL * device_sms()) g = 16LL * device_sms();
+  hs_launch(double_layer_dense_kernel, (unsigned)g, 256, (size_t)q * sizeof(int2), s, A, d, D, cplx, out);
   return cudaGetLastError();
 }
 
@@ -365,8 +442,8 @@ cudaError_t launch_from_hermitian(const double* t, int D, bool graded, double* o
 
 cudaError_t launch_rotate_dense_to_blocks(const double* a, int D, double* out,
                                           unsigned long long* maxes, cudaStream_t s) {
-  const long long q = (long long)D * D;
-  hs_launch(rotate_dense_kernel, grid_for(q * q * q * q), 256, 0, s, a, D, out, maxes);
+  const long long ne = (long long)D * (D + 1) / 2;
+  hs_launch(rotate_dense_kernel, grid_for(ne * ne * ne * ne), 256, (size_t)ne * sizeof(int2), s, a, D, out, maxes);
   return cudaGetLastError();
 }
 
