@@ -303,24 +303,16 @@ HS_HD bool f32_widen_fast(uint32_t f, unsigned long long& out) {
 //   X = sum_{i=1..7} d_i 256^(7 - i),  d_i in [-128, 127] (d_1 up to 128),
 // so that slice i holds the integers d_i, exact in BF16.
 
-// X of x for a row whose largest exponent field is emax (x finite, emax >= 1).
-HS_HD long long slice_fixed(double x, int emax) {
-  const unsigned long long b = f64_bits(x);
-  int E = (int)((b >> 52) & 0x7FF);
-  unsigned long long m = b & 0xFFFFFFFFFFFFFull;
-  if (E)
-    m |= 1ull << 52;
-  else
-    E = 1;  // subnormal
-  const int d = emax - E;  // >= 0
-  unsigned long long v;
-  if (d <= 2) {
-    v = m << (2 - d);
-  } else {
-    const int r = d - 2;
-    v = r <= 54 ? (m + (1ull << (r - 1))) >> r : 0ull;
-  }
-  return (b >> 63) ? -(long long)v : (long long)v;
+// X of the double with bits b for a row whose largest exponent field is emax:
+// the mantissa, aligned to bit 63, shifted right and rounded (halves up in
+// magnitude). Zeros and subnormals give 0 through their distance from emax
+// (rows with emax below 100 are not handled by the slices).
+HS_HD long long slice_fixed(unsigned long long b, int emax) {
+  const int s = 8 + emax - (int)((b >> 52) & 0x7FF);
+  const unsigned long long m = (b << 11) | (1ull << 63);
+  const unsigned long long v = s < 64 ? ((m >> s) + 1) >> 1 : 0ull;
+  const long long sg = (long long)b >> 63;
+  return ((long long)v ^ sg) - sg;
 }
 
 // Y = X + sum of 128 at the six lower digits: d_i = byte (7 - i) of Y minus 128

@@ -424,10 +424,12 @@ struct SplitOps {
   SplitOp op[kMaxSplit];
 };
 
-__device__ __forceinline__ double sl_at(const SlMat& m, long long roff, int k) {
+// Bits of entry k of a row, its sign flipped where the source is negated (as an
+// integer: negating a double takes the FP64 pipe).
+__device__ __forceinline__ unsigned long long sl_at(const SlMat& m, long long roff, int k) {
   const int s = k >= m.kseg;
-  const double x = (s ? m.p[1] + roff - m.kseg : m.p[0] + roff)[k];
-  return m.neg[s] ? -x : x;
+  const double* p = s ? m.p[1] + roff - m.kseg : m.p[0] + roff;
+  return f64_bits(p[k]) ^ ((unsigned long long)m.neg[s] << 63);
 }
 
 // Float of digit i times 2^(-8 (i - 1)) from the biased value (exact, its upper
@@ -441,73 +443,129 @@ __device__ __forceinline__ uint32_t digit_bits(unsigned lo, unsigned hi, int i) 
   return __float_as_uint(fmaf(m, s, -(8388608.f + 128.f) * s));
 }
 
-// One warp per row: the largest exponent, then the seven digits of every
-// entry, two columns a lane (four-byte stores, 128 bytes a warp and plane).
-// Bound by memory: 8 bytes read and 14 written per entry. NR > 0: rows of at
-// most 64 NR entries, held in registers between the two passes (every load of
-// a row in flight at once); NR = 0: any length, read twice.
+// The digits of 8 consecutive columns are 16 bytes of a plane's row, one thread's
+// work: 64 bytes read, seven 16-byte stores. T threads share a row (T a power of
+// two up to 32, or the whole block of 256), each with NR pieces held in registers
+// between the row's largest exponent and its digits, so a row is read once; NR =
+// 0 reads it twice, for rows too long for the registers. Bound by memory (8
+// bytes read and 14 written per entry): 10368 x 666 takes 31 us (4-byte stores
+// and a warp per row: 67), 20736 x 5184 0.43 ms (1.6).
+__device__ __forceinline__ void sl_load(const SplitOp& P, bool vec, long long roff, int k,
+                                        unsigned long long (&x)[8]) {
+  if (vec) {
+    const int s = k >= P.m.kseg;
+    const double* p = (s ? P.m.p[1] + roff - P.m.kseg : P.m.p[0] + roff) + k;
+    const unsigned long long flip = (unsigned long long)P.m.neg[s] << 63;
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+      const ulonglong2 d =
+          k + j < P.K ? *reinterpret_cast<const ulonglong2*>(p + j) : make_ulonglong2(0ull, 0ull);
+      x[j] = d.x ^ flip;
+      x[j + 1] = d.y ^ flip;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) x[j] = k + j < P.K ? sl_at(P.m, roff, k + j) : 0ull;
+  }
+}
+
+__device__ __forceinline__ unsigned long long sl_mag(const unsigned long long (&x)[8], unsigned long long mag) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) mag = max(mag, x[j] & 0x7FFFFFFFFFFFFFFFull);
+  return mag;
+}
+
+__device__ __forceinline__ void sl_put(const SplitOp& P, unsigned char* row, int rr, int k, int emax,
+                                       const unsigned long long (&x)[8]) {
+  const size_t plane = (size_t)P.block * ROW_BYTES;
+  unsigned char* o = row + (size_t)(k / KC) * NS * plane + (((k % KC) / 8) ^ ((rr >> 1) & 3)) * 16;
+  unsigned lo[8], hi[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const long long y = slice_bias(slice_fixed(x[j], emax));
+    lo[j] = (unsigned)y;
+    hi[j] = (unsigned)((unsigned long long)y >> 32);
+  }
+#pragma unroll
+  for (int i = 1; i <= NS; ++i) {
+    uint4 w;
+    w.x = __byte_perm(digit_bits(lo[0], hi[0], i), digit_bits(lo[1], hi[1], i), 0x7632);
+    w.y = __byte_perm(digit_bits(lo[2], hi[2], i), digit_bits(lo[3], hi[3], i), 0x7632);
+    w.z = __byte_perm(digit_bits(lo[4], hi[4], i), digit_bits(lo[5], hi[5], i), 0x7632);
+    w.w = __byte_perm(digit_bits(lo[6], hi[6], i), digit_bits(lo[7], hi[7], i), 0x7632);
+    *reinterpret_cast<uint4*>(o + (i - 1) * plane) = w;
+  }
+}
+
 template <int NR>
-__global__ void __launch_bounds__(256) slice_split_kernel(const __grid_constant__ SplitOps ops) {
+__global__ void __launch_bounds__(256) slice_split_kernel(const __grid_constant__ SplitOps ops, int T) {
   hs_pdl_enter();
   const SplitOp& P = ops.op[blockIdx.y];
-  const int lane = threadIdx.x % 32;
-  const int Kp = P.steps * KC, plane = P.block * ROW_BYTES;
-  // 16-byte loads: one source, rows of even length on even strides
-  const bool vec = P.m.nseg == 1 && P.K % 2 == 0 && P.m.ld % 2 == 0 &&
-                   (reinterpret_cast<uintptr_t>(P.m.p[0]) & 15) == 0;
-  for (int r = blockIdx.x * 8 + threadIdx.x / 32; r < P.m.rows; r += gridDim.x * 8) {
-    const long long roff = (long long)r * P.m.ld;
-    double x[NR > 0 ? NR : 1][2];
+  const int Kp = P.steps * KC;
+  // 16-byte loads: even strides and lengths, sources aligned and changing between pieces
+  const bool vec = P.K % 2 == 0 && P.m.ld % 2 == 0 && (reinterpret_cast<uintptr_t>(P.m.p[0]) & 15) == 0 &&
+                   (P.m.nseg == 1 || (P.m.kseg % 8 == 0 && (reinterpret_cast<uintptr_t>(P.m.p[1]) & 15) == 0));
+  __shared__ unsigned long long red[8];
+  const int per = 256 / T, t = threadIdx.x % T;  // rows of the block at a time, thread within the row
+  // the whole block runs the same number of turns (its barriers)
+  for (int r0 = blockIdx.x * per; r0 < P.m.rows; r0 += gridDim.x * per) {
+    const int r = r0 + threadIdx.x / T;
+    const bool in = r < P.m.rows;
+    const long long roff = (long long)(in ? r : 0) * P.m.ld;
+    unsigned long long x[NR > 0 ? NR : 1][8];
     unsigned long long mag = 0;  // largest |bits|: its exponent field is the row's
-    constexpr unsigned long long kMag = 0x7FFFFFFFFFFFFFFFull;
     if (NR > 0) {
 #pragma unroll
       for (int i = 0; i < NR; ++i) {
-        const int k = 64 * i + 2 * lane;
-        if (vec) {
-          const double2 d = k < P.K ? *reinterpret_cast<const double2*>(P.m.p[0] + roff + k) : make_double2(0.0, 0.0);
-          x[i][0] = P.m.neg[0] ? -d.x : d.x;
-          x[i][1] = P.m.neg[0] ? -d.y : d.y;
+        const int k = 8 * (t + i * T);
+        if (in && k < P.K) {
+          sl_load(P, vec, roff, k, x[i]);
         } else {
-          x[i][0] = k < P.K ? sl_at(P.m, roff, k) : 0.0;
-          x[i][1] = k + 1 < P.K ? sl_at(P.m, roff, k + 1) : 0.0;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[i][j] = 0ull;
         }
       }
 #pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        mag = max(mag, f64_bits(x[i][0]) & kMag);
-        mag = max(mag, f64_bits(x[i][1]) & kMag);
-      }
+      for (int i = 0; i < NR; ++i) mag = sl_mag(x[i], mag);
     } else {
-      for (int k = lane; k < P.K; k += 32) mag = max(mag, f64_bits(sl_at(P.m, roff, k)) & kMag);
+      for (int k = 8 * t; k < P.K; k += 8 * T) {
+        sl_load(P, vec, roff, k, x[0]);
+        mag = sl_mag(x[0], mag);
+      }
     }
-    for (int o = 16; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
-    const int ef = (int)(mag >> 52), emax = ef > 0 ? ef : 1;
-    if (lane == 0) {
+    for (int o = (T < 32 ? T : 32) / 2; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+    if (T > 32) {
+      __syncthreads();
+      if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = mag;
+      __syncthreads();
+#pragma unroll
+      for (int w = 0; w < 8; ++w) mag = max(mag, red[w]);
+    }
+    if (!in) continue;
+    // zero rows and rows of the smallest scales (marked) get zero digits
+    const int ef = (int)(mag >> 52), emax = ef >= 100 ? ef : 0x7FF;
+    if (t == 0) {
       const int e = ef - 1022;
       P.exps[r] = mag == 0 ? 0 : (ef == 0x7FF || e > 500 || e < -400) ? kSpecial : e;
     }
     const int rb = r / P.block, rr = r - rb * P.block;
-    unsigned char* out = P.planes + (size_t)rb * P.steps * NS * plane + rr * ROW_BYTES;
-    auto put = [&](int k, double x0, double x1) {
-      unsigned char* o = out + (size_t)(k / KC) * NS * plane + ((((k % KC) / 8) ^ ((rr >> 1) & 3)) * 16) + (k % 8) * 2;
-      const long long y0 = slice_bias(slice_fixed(x0, emax)), y1 = slice_bias(slice_fixed(x1, emax));
-      const unsigned l0 = (unsigned)y0, h0 = (unsigned)((unsigned long long)y0 >> 32);
-      const unsigned l1 = (unsigned)y1, h1 = (unsigned)((unsigned long long)y1 >> 32);
-#pragma unroll
-      for (int i = 1; i <= NS; ++i)
-        *reinterpret_cast<uint32_t*>(o + (i - 1) * plane) =
-            __byte_perm(digit_bits(l0, h0, i), digit_bits(l1, h1, i), 0x7632);
-    };
+    unsigned char* row = P.planes + (size_t)rb * P.steps * NS * P.block * ROW_BYTES + rr * ROW_BYTES;
     if (NR > 0) {
 #pragma unroll
       for (int i = 0; i < NR; ++i) {
-        const int k = 64 * i + 2 * lane;
-        if (k < Kp) put(k, x[i][0], x[i][1]);
+        const int k = 8 * (t + i * T);
+        if (k < Kp) sl_put(P, row, rr, k, emax, x[i]);
       }
     } else {
-      for (int k = 2 * lane; k < Kp; k += 64)
-        put(k, k < P.K ? sl_at(P.m, roff, k) : 0.0, k + 1 < P.K ? sl_at(P.m, roff, k + 1) : 0.0);
+      for (int k = 8 * t; k < Kp; k += 8 * T) {
+        if (k < P.K) {
+          sl_load(P, vec, roff, k, x[0]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) x[0][j] = 0ull;
+        }
+        sl_put(P, row, rr, k, emax, x[0]);
+      }
     }
   }
 }
@@ -598,17 +656,26 @@ cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* pro
     tiles += (int)t;
   }
   const int sms = device_sms();
-  int gx = (rmax + 7) / 8;
-  if (gx > sms * 16) gx = sms * 16;
+  // threads per row: one piece of 8 columns each up to a warp, then up to four,
+  // then the block with up to three
+  const int pieces = steps_of(kmax) * (KC / 8);
+  int T = 4;
+  while (T < 32 && T < pieces) T *= 2;
+  if (pieces > 128) T = 256;
+  const int nr = (pieces + T - 1) / T, per = 256 / T;
+  int gx = (rmax + per - 1) / per;
+  if (gx > sms * 32) gx = sms * 32;
   const dim3 grid((unsigned)gx, (unsigned)nmat);
-  if (kmax <= 64)
-    hs_launch(slice_split_kernel<1>, grid, 256, 0, s, ops);
-  else if (kmax <= 256)
-    hs_launch(slice_split_kernel<4>, grid, 256, 0, s, ops);
-  else if (kmax <= 768)
-    hs_launch(slice_split_kernel<12>, grid, 256, 0, s, ops);
+  if (nr == 1)
+    hs_launch(slice_split_kernel<1>, grid, 256, 0, s, ops, T);
+  else if (nr == 2)
+    hs_launch(slice_split_kernel<2>, grid, 256, 0, s, ops, T);
+  else if (nr == 3)
+    hs_launch(slice_split_kernel<3>, grid, 256, 0, s, ops, T);
+  else if (nr == 4 && T == 32)
+    hs_launch(slice_split_kernel<4>, grid, 256, 0, s, ops, T);
   else
-    hs_launch(slice_split_kernel<0>, grid, 256, 0, s, ops);
+    hs_launch(slice_split_kernel<0>, grid, 256, 0, s, ops, T);
   const cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(gemm_sl_kernel), SMEM);
   if (e != cudaSuccess) return e;
   hs_launch(gemm_sl_kernel, (unsigned)(tiles < sms ? tiles : sms), NT, SMEM, s, g, tiles, accumulate, err);

@@ -14,14 +14,14 @@ int main() {
   std::mt19937_64 g(1);
   long bad = 0;
   for (long t = 0; t < 2000000; ++t) {
-    const int emax = 1 + (int)(g() % 2046);
-    // exponents from emax down to 80 below it (subnormals at the bottom), and the largest mantissa
-    const int drop = (int)(g() % 80), ef = emax - drop > 0 ? emax - drop : 0;
+    const int emax = 100 + (int)(g() % 1946);
+    // exponents from emax down to 80 below it, subnormals and zeros, and the largest and smallest mantissas
+    const int ef = t % 11 == 0 ? 0 : emax - (int)(g() % 80);
     unsigned long long m = g() & 0xFFFFFFFFFFFFFull;
     if (t % 13 == 0) m = 0xFFFFFFFFFFFFFull;
     if (t % 17 == 0) m = 0;
     const double x = f64_from_bits((g() & (1ull << 63)) | ((unsigned long long)ef << 52) | m);
-    const long long X = slice_fixed(x, emax), Y = slice_bias(X);
+    const long long X = slice_fixed(f64_bits(x), emax), Y = slice_bias(X);
     long long back = 0;
     for (int i = 1; i <= 7; ++i) {
       const int d = slice_digit(Y, i);
