@@ -384,6 +384,10 @@ __global__ void cheb_step_pair_kernel(double* __restrict__ Y, const double* __re
 // accumulates V only for its slice of the eigenvector components: the work of
 // a round is shared-memory bound, and V is the larger half of it. A is kept as
 // its upper triangle, so a 2 x 2 block of a round is read and written once.
+// A round is two phases between barriers: the rotations (a chain of divisions
+// and square roots in two or three warps) beside the last round's update of V,
+// then the update of A. The table of a round carries its pairs' indices, so that
+// a block costs two 16-byte loads instead of two searches of the ordering.
 constexpr int kMaxSweeps = 40;
 constexpr int kJacobiCtas = 8;
 
@@ -435,7 +439,8 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
   const int i0 = g * mc, nc = max(0, min(m, i0 + mc) - i0);
   float* A = shj;                                           // upper triangle of m x ld
   float* Vt = A + m * ld;                                   // m x mc: Vt[j * mc + i] = component i0 + i of vector j
-  float2* cs = reinterpret_cast<float2*>(Vt + ((m * mc + 1) & ~1));  // (cos, sin) per pair (8-byte aligned)
+  // two tables of (cos, sin, p | q << 16) per pair: this round's and the last one's
+  float4* rot = reinterpret_cast<float4*>(shj + ((m * ld + m * mc + 3) & ~3));
   const int M = (m + 1) & ~1;  // even player count (index m is a dummy when m is odd)
   const int npair = M / 2;
   const float kRelTol = fmaxf(4e-7f, sqrtf((float)m) * 6e-8f);
@@ -476,14 +481,15 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
     }
   }
   // this thread's V entries: pair b, local component i (consecutive threads
-  // take consecutive components)
+  // take consecutive components); the warps that compute the rotations have none
+  const int rw = (npair + 31) & ~31;
   int ven[kVPerThread];
   int nven = 0;
 #pragma unroll
   for (int t = 0; t < kVPerThread; ++t) {
-    const int f = threadIdx.x + t * blockDim.x;
+    const int f = (int)threadIdx.x - rw + t * ((int)blockDim.x - rw);
     ven[t] = -1;
-    if (nc > 0 && f < npair * nc) {
+    if ((int)threadIdx.x >= rw && nc > 0 && f < npair * nc) {
       ven[t] = ((f / nc) << 16) | (f % nc);
       nven = t + 1;
     }
@@ -493,12 +499,32 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
   for (int w = 0; w < (int)(blockDim.x >> 5); ++w) dmax = fmaxf(dmax, dmax_part[w]);
   // off-diagonal entries below this are rounding noise of the FP32 matrix
   const float abs_floor = 1e-7f * dmax;
+  // V <- V J of one round on this CTA's components
+  auto update_v = [&](const float4* rt) {
+#pragma unroll
+    for (int t = 0; t < kVPerThread; ++t) {
+      if (t >= nven) break;
+      const int b = ven[t] >> 16, i = ven[t] & 0xffff;
+      const float4 rb_ = rt[b];
+      if (rb_.x == 1.f && rb_.y == 0.f) continue;  // no rotation (or the dummy pair)
+      const unsigned pq = __float_as_uint(rb_.z);
+      const int p = (int)(pq & 0xffff) * mc + i, q = (int)(pq >> 16) * mc + i;
+      const float vp = Vt[p], vq = Vt[q];
+      Vt[p] = rb_.x * vp - rb_.y * vq;
+      Vt[q] = rb_.y * vp + rb_.x * vq;
+    }
+  };
   bool converged = false;
+  int buf = 0;
+  bool pending = false;  // the last round's rotations (table 1 - buf) have not reached V yet
   for (int sweep = 0; sweep < kMaxSweeps && !converged; ++sweep) {
     int nrot = 0;  // rotations in this sweep (the same in every thread)
     for (int r = 0; r < M - 1; ++r) {
+      // the first warps find this round's rotations, a chain of latencies, while
+      // the others apply the last round's to V
       int rotates = 0;
-      for (int k = threadIdx.x; k < npair; k += blockDim.x) {
+      if ((int)threadIdx.x < npair) {
+        const int k = threadIdx.x;
         const int2 pq = rr_pair(k, r, M);
         float c = 1.f, sn = 0.f;
         if (pq.y < m) {
@@ -513,8 +539,11 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
             rotates = 1;
           }
         }
-        cs[k] = make_float2(c, sn);
+        rot[buf * npair + k] = make_float4(c, sn, __uint_as_float((unsigned)pq.x | (unsigned)pq.y << 16), 0.f);
+      } else if (pending) {
+        update_v(rot + (1 - buf) * npair);
       }
+      pending = false;
       const int rrot = __syncthreads_count(rotates);
       if (rrot == 0) continue;  // nothing rotates in this round (block-uniform)
       nrot += rrot;
@@ -525,10 +554,11 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
       for (int t = 0; t < kBlkPerThread; ++t) {
         if (t >= nblk) break;
         const int a = blk[t] >> 16, b = blk[t] & 0xffff;
-        const float2 ra_ = cs[a], rb_ = cs[b];
+        const float4 ra_ = rot[buf * npair + a], rb_ = rot[buf * npair + b];
         // neither pair rotates: the block stays as it is
         if (ra_.x == 1.f && ra_.y == 0.f && rb_.x == 1.f && rb_.y == 0.f) continue;
-        const int2 ia = rr_pair(a, r, M), ib = rr_pair(b, r, M);
+        const unsigned pa = __float_as_uint(ra_.z), pb = __float_as_uint(rb_.z);
+        const int2 ia = make_int2((int)(pa & 0xffff), (int)(pa >> 16)), ib = make_int2((int)(pb & 0xffff), (int)(pb >> 16));
         const bool ra = ia.y < m, rb = ib.y < m;
         // (pa, pb), (pa, qb), (qa, pb), (qa, qb) at their upper positions
         const int e00 = min(ia.x, ib.x) * ld + max(ia.x, ib.x);
@@ -549,22 +579,14 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
         if (ra && a != b) A[e10] = n10;
         if (ra && rb) A[e11] = n11;
       }
-      // V <- V J on this CTA's components
-#pragma unroll
-      for (int t = 0; t < kVPerThread; ++t) {
-        if (t >= nven) break;
-        const int b = ven[t] >> 16, i = ven[t] & 0xffff;
-        const float2 rb_ = cs[b];
-        if (rb_.x == 1.f && rb_.y == 0.f) continue;  // no rotation (or the dummy pair)
-        const int2 ib = rr_pair(b, r, M);
-        const float vp = Vt[ib.x * mc + i], vq = Vt[ib.y * mc + i];
-        Vt[ib.x * mc + i] = rb_.x * vp - rb_.y * vq;
-        Vt[ib.y * mc + i] = rb_.y * vp + rb_.x * vq;
-      }
+      pending = true;
+      buf = 1 - buf;
       __syncthreads();
     }
     converged = nrot == 0;  // a sweep without a rotation: every A_pq is negligible
   }
+  if (pending) update_v(rot + (1 - buf) * npair);
+  __syncthreads();
   if (!converged && g == 0 && threadIdx.x == 0) atomicExch(status, 1);
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   // ascending order by rank (ties by index); vectors as columns, column-major
@@ -584,7 +606,7 @@ __global__ void __launch_bounds__(1024) jacobi_eig_kernel(float* __restrict__ A0
 
 size_t jacobi_smem_bytes(int m) {
   const int mc = (m + kJacobiCtas - 1) / kJacobiCtas;
-  return (size_t)(m * (m + 1) + ((m * mc + 1) & ~1)) * sizeof(float) + (size_t)((m + 1) / 2 + 1) * sizeof(float2);
+  return (size_t)(m * (m + 1) + m * mc + 8) * sizeof(float) + (size_t)(2 * ((m + 1) / 2)) * sizeof(float4);
 }
 
 cudaError_t launch_jacobi_eig_pair(float* A0, int m0, float* w0, float* A1, int m1, float* w1, int* status,
@@ -594,7 +616,8 @@ cudaError_t launch_jacobi_eig_pair(float* A0, int m0, float* w0, float* A1, int 
   // m <= kMaxSub keeps the (m/2)(m/2 + 1)/2 blocks of a round within kBlkPerThread per thread
   // and the (m/2) ceil(m / kJacobiCtas) V entries within kVPerThread
   static_assert((kMaxSub / 2 + 1) * (kMaxSub / 2 + 2) / 2 <= kBlkPerThread * 1024, "block grid too large");
-  static_assert((kMaxSub / 2 + 1) * ((kMaxSub + kJacobiCtas - 1) / kJacobiCtas) <= kVPerThread * 1024,
+  static_assert((kMaxSub / 2 + 1) * ((kMaxSub + kJacobiCtas - 1) / kJacobiCtas) <=
+                    kVPerThread * (1024 - ((kMaxSub / 2 + 31) & ~31)),
                 "V slice too large");
   if (m > kMaxSub) return cudaErrorInvalidValue;
   // set once per device
