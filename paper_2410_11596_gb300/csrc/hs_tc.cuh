@@ -93,18 +93,13 @@ __device__ __forceinline__ uint32_t elect_one() {
   return r;
 }
 
-// mma_commit by the lane with leader != 0.
+// Arrive on bar when the MMAs issued so far are done, by the lane with leader != 0.
 __device__ __forceinline__ void mma_commit_by(uint32_t leader, uint32_t bar) {
   asm volatile(
       "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
       " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
       "r"(leader)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
 }
 
 __device__ __forceinline__ void fence_before() {

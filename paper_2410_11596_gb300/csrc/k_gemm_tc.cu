@@ -90,16 +90,10 @@ __device__ __forceinline__ int ps_co(const PsDesc& D, int tr, int tc, int k) {
 }
 
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row core
-// groups 1024 bytes apart (rows are 128 bytes), descriptor version 1.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;            // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset
-  d |= (uint64_t)1 << 46;            // version
-  d |= (uint64_t)2 << 61;            // 128-byte swizzle
-  return d;
-}
+// groups 1024 bytes apart (rows are 128 bytes), descriptor version 1. The upper
+// word is a constant, the lower one holds the address in 16-byte units.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3FFFF) >> 4) | (1u << 16); }
 
 // Instruction descriptor of kind::tf32 / kind::f16: D = f32, A/B format
 // (2 = tf32, 1 = bf16), both K-major, N = BN, M = BM.
@@ -108,17 +102,19 @@ __host__ __device__ constexpr uint32_t idesc(uint32_t fmt) {
 }
 
 template <int EB>
-__device__ __forceinline__ void mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void mma(uint32_t leader, uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t acc) {
   if (EB == 4) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::
-            "r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc(2)), "r"(acc));
+        "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+        " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+        " @q tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(kDescHi), "r"(idesc(2)), "r"(acc), "r"(leader));
   } else {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::
-            "r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc(1)), "r"(acc));
+        "{\n .reg .pred p, q;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n setp.ne.b32 q, %6, 0;\n"
+        " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+        "r"(a), "r"(b), "r"(kDescHi), "r"(idesc(1)), "r"(acc), "r"(leader));
   }
 }
 
@@ -178,7 +174,7 @@ __global__ void __launch_bounds__(NT, 1) gemm_tc_kernel(const __grid_constant__ 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;  // warp: uniform
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -239,49 +235,50 @@ __global__ void __launch_bounds__(NT, 1) gemm_tc_kernel(const __grid_constant__ 
       for (long long j = it > K::STAGES ? it - K::STAGES : 0; j < it; ++j)
         mbar_drain(smem_u32(&full[j % K::STAGES]), (uint32_t)((j / K::STAGES) & 1));
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer ----
+  } else if (warp == 1) {
+    // ---- MMA issuer: the whole warp, one elected lane's instructions ----
+    const uint32_t leader = elect_one();
+    auto wait = [&](uint64_t* bar, long long n, int code) {
+      return (bool)__all_sync(0xffffffffu, mbar_wait(smem_u32(bar), (uint32_t)(n & 1), abort_flag, err, code));
+    };
     long long it = 0;
-    bool any = false;
+    bool any = false, ok = true;
     int local = 0;
-    for (int t = blockIdx.x; t < total_tiles && !*abort_flag; t += gridDim.x, ++local) {
+    for (int t = blockIdx.x; ok && t < total_tiles; t += gridDim.x, ++local) {
       const TileRef r = tile_of(g, t);
       const int ktiles = g.p[r.pi].Kp / K::K_PER_TILE;
       const int buf = local & 1, use = local >> 1;
-      if (use > 0 && !mbar_wait(smem_u32(&tempty[buf]), (uint32_t)((use - 1) & 1), abort_flag, err, 4)) break;
+      if (use > 0) ok = wait(&tempty[buf], use - 1, 4);
+      if (!ok) break;
       fence_after();
       const uint32_t d = tmem + (uint32_t)buf * K::ACC_COLS;
-      bool ok = true;
       for (int kt = 0; kt < ktiles; ++kt) {
         const int s = (int)(it % K::STAGES);
-        const long long n = it / K::STAGES;
-        if (!mbar_wait(smem_u32(&full[s]), (uint32_t)(n & 1), abort_flag, err, 2)) {
-          ok = false;
-          break;
-        }
+        ok = wait(&full[s], it / K::STAGES, 2);
+        if (!ok) break;
         fence_after();
         const uint32_t st = smem_u32(smem + s * K::STAGE_BYTES);
-        const uint64_t a_hi = sdesc(st), b_hi = sdesc(st + TILE_BYTES);
-        const uint64_t a_lo = sdesc(st + 2 * TILE_BYTES), b_lo = sdesc(st + 3 * TILE_BYTES);
+        const uint32_t a_hi = desc_lo(st), b_hi = desc_lo(st + TILE_BYTES);
+        const uint32_t a_lo = desc_lo(st + 2 * TILE_BYTES), b_lo = desc_lo(st + 3 * TILE_BYTES);
 #pragma unroll
         for (int kk = 0; kk < ROW_BYTES / 32; ++kk) {
-          const uint64_t off = (uint64_t)((kk * 32) >> 4);
+          const uint32_t off = (kk * 32) >> 4;
           const uint32_t acc = (kt | kk) != 0;
-          mma<EB>(d, a_hi + off, b_hi + off, acc);
+          mma<EB>(leader, d, a_hi + off, b_hi + off, acc);
           if (NPASS == 3) {
-            mma<EB>(d + BN, a_hi + off, b_lo + off, acc);
-            mma<EB>(d + BN, a_lo + off, b_hi + off, 1);
+            mma<EB>(leader, d + BN, a_hi + off, b_lo + off, acc);
+            mma<EB>(leader, d + BN, a_lo + off, b_hi + off, 1);
           }
         }
         any = true;
-        mma_commit(smem_u32(&empty[s]));
+        mma_commit_by(leader, smem_u32(&empty[s]));
         ++it;
       }
       if (!ok) break;
-      mma_commit(smem_u32(&tfull[buf]));  // arrives once this tile's MMAs are done
+      mma_commit_by(leader, smem_u32(&tfull[buf]));  // arrives once this tile's MMAs are done
     }
-    if (*abort_flag && any) {
-      mma_commit(smem_u32(drain));
+    if (!ok && any) {
+      mma_commit_by(leader, smem_u32(drain));
       mbar_drain(smem_u32(drain), 0);
     }
   } else if (warp >= 2) {
