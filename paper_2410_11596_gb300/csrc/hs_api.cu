@@ -379,8 +379,9 @@ hs_status tc_split_f32(hs_ctx ctx, hs_precision prec, const Z2Mat& src_layout, c
 
 // Sizes the split buffers of the padded operand layout P and zeroes their K
 // padding unless the last split into them had the same layout (a split
-// writes every entry of the layout but none of the padding).
-hs_status split_dest(hs_ctx ctx, hs_precision prec, const Z2Mat& P, DBuf& hi, DBuf& lo) {
+// writes every entry of the layout but none of the padding); with pads, the
+// zeroing is left to the split kernel.
+hs_status split_dest(hs_ctx ctx, hs_precision prec, const Z2Mat& P, DBuf& hi, DBuf& lo, SplitPads* pads = nullptr) {
   const int eb = tc_elem_bytes(prec);
   const size_t nb = (size_t)z2_elems(P) * eb;
   HS_TRY(hi.ensure(nb));
@@ -395,6 +396,13 @@ hs_status split_dest(hs_ctx ctx, hs_precision prec, const Z2Mat& P, DBuf& hi, DB
     for (int p = 0; p < 2; ++p) {
       const long long rows = z2_rows(P, p), cols = z2_cols(P, p), ld = z2_ld(P, p);
       if (rows == 0 || ld == cols) continue;
+      if (pads) {
+        pads->rows[p] = (unsigned)rows;
+        pads->width[p] = (unsigned)(ld - cols);
+        pads->off[p] = z2_block_off(P, p) + cols;
+        pads->ld[p] = ld;
+        continue;
+      }
       const size_t off = (size_t)(z2_block_off(P, p) + cols) * eb;
       for (DBuf* b : {&hi, &lo})
         HS_CUDA(cudaMemset2DAsync(static_cast<char*>(b->p) + off, (size_t)ld * eb, 0, (size_t)(ld - cols) * eb,
@@ -409,14 +417,16 @@ hs_status tc_split_any(hs_ctx ctx, hs_precision prec, const Z2Mat& src_layout, c
                        std::initializer_list<int> perm, const void* src, bool src_f32, DBuf& hi, DBuf& lo) {
   const Z2Mat P = mat(layout.r, layout.c, tc_pad(prec));
   PhaseScope ps(ctx, HS_PHASE_PERMUTE);
-  HS_TRY(split_dest(ctx, prec, P, hi, lo));
   int pm[kMaxLegs] = {0}, i = 0;
   for (int v : perm) pm[i++] = v;
   const PermPlan& plan = cached_plan(ctx, src_layout, P, pm);
+  SplitPads pads;
+  HS_TRY(split_dest(ctx, prec, P, hi, lo, plan.nbox > 0 ? &pads : nullptr));
   if (src_f32)
-    HS_CUDA(launch_permute_split_f32(plan, static_cast<const float*>(src), hi.p, lo.p, tc_mode(prec), ctx->stream));
+    HS_CUDA(launch_permute_split_f32(plan, static_cast<const float*>(src), hi.p, lo.p, tc_mode(prec), ctx->stream,
+                                     pads));
   else
-    HS_CUDA(launch_permute_split(plan, static_cast<const double*>(src), hi.p, lo.p, tc_mode(prec), ctx->stream));
+    HS_CUDA(launch_permute_split(plan, static_cast<const double*>(src), hi.p, lo.p, tc_mode(prec), ctx->stream, pads));
   if (plan.nbox > 0) ctx->launches += 1;
   return HS_OK;
 }

@@ -320,20 +320,26 @@ double gemm_flops(const GemmGroup& g);
 
 cudaError_t launch_permute_f64(const PermPlan& plan, const double* in, double* out, double scale,
                                cudaStream_t s);
+// The padding columns of a split operand's two blocks: rows rows of width
+// elements each, ld elements apart, from element off (width or rows 0: none).
+struct SplitPads {
+  unsigned rows[2] = {0, 0}, width[2] = {0, 0};
+  long long off[2] = {0, 0}, ld[2] = {0, 0};
+};
 // Same permutation, writing the operand split for the tensor cores:
 // mode 1: hi = tf32(x), lo = fp32(x - hi) as float; mode 2: bf16 hi/lo pair.
-// The padded columns of `out` must have been zeroed by the caller.
+// The padded columns of `out` are zeroed where pads says so.
 // FP32 sources (values that came out of the tensor-core GEMMs' FP32 accumulators).
 cudaError_t launch_permute_f32(const PermPlan& plan, const float* in, float* out, cudaStream_t s);
 cudaError_t launch_permute_split_f32(const PermPlan& plan, const float* in, void* hi, void* lo, int mode,
-                                     cudaStream_t s);
+                                     cudaStream_t s, const SplitPads& pads = SplitPads());
 // FP32 values of a TF32x3-split block pair (padded rows of ld0/ld1 elements,
 // block 1 at element off1) into out, tightly packed, block 1 after block 0.
 cudaError_t launch_join_split_f32(const void* hi, const void* lo, long long rows0, long long cols0, long long ld0,
                                   long long off1, long long rows1, long long cols1, long long ld1, float* out,
                                   cudaStream_t s);
 cudaError_t launch_permute_split(const PermPlan& plan, const double* in, void* hi, void* lo, int mode,
-                                 cudaStream_t s);
+                                 cudaStream_t s, const SplitPads& pads = SplitPads());
 
 // Split a row-major FP64 matrix [rows, cols] (row stride ld_src) into padded
 // hi/lo operands [rows, ld_dst] (zeros in columns cols..ld_dst-1); mode as above.

@@ -496,10 +496,30 @@ __device__ __forceinline__ void store_split(double x, void* hi, void* lo, long l
   }
 }
 
+// The K padding of the operand's block rows is zeroed here too (the first plan
+// row of CTAs): as memsets between the launches it cost more than the split, since
+// a memset waits for the kernel before it and the next kernel for the memset.
 template <int MODE, int NB, class T>
-__global__ void permute_split_kernel(PlanArg<NB> plan, const T* __restrict__ in, void* __restrict__ hi,
-                                     void* __restrict__ lo) {
+__global__ void permute_split_kernel(PlanArg<NB> plan, SplitPads pads, const T* __restrict__ in,
+                                     void* __restrict__ hi, void* __restrict__ lo) {
   hs_pdl_enter();
+  if (blockIdx.y == 0) {
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const unsigned w = pads.width[p], total = pads.rows[p] * w;
+      for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
+        const unsigned row = e / w;
+        const long long at = pads.off[p] + (long long)row * pads.ld[p] + (e - row * w);
+        if (MODE == 1) {
+          static_cast<uint32_t*>(hi)[at] = 0u;
+          static_cast<uint32_t*>(lo)[at] = 0u;
+        } else {
+          static_cast<uint16_t*>(hi)[at] = 0;
+          static_cast<uint16_t*>(lo)[at] = 0;
+        }
+      }
+    }
+  }
   const Box& b = plan.box[blockIdx.y];
   if (b.plane > 0) {
     permute_planes(b, in, [&](unsigned o, T v) { store_split<MODE>(v, hi, lo, (long long)o); });
@@ -540,7 +560,8 @@ __global__ void permute_split_kernel(PlanArg<NB> plan, const T* __restrict__ in,
 }
 
 template <class T>
-cudaError_t launch_permute_split_t(const PermPlan& plan, const T* in, void* hi, void* lo, int mode, cudaStream_t s) {
+cudaError_t launch_permute_split_t(const PermPlan& plan, const T* in, void* hi, void* lo, int mode, cudaStream_t s,
+                                   const SplitPads& pads) {
   if (plan.nbox == 0) return cudaSuccess;
   const long long maxc = max_work(plan);
   long long gx = (maxc + 255) / 256;
@@ -551,9 +572,9 @@ cudaError_t launch_permute_split_t(const PermPlan& plan, const T* in, void* hi, 
     PlanArg<NB> arg;
     for (int i = 0; i < plan.nbox; ++i) arg.box[i] = plan.box[i];
     if (mode == 1)
-      hs_launch(permute_split_kernel<1, NB, T>, grid, 256, 0, s, arg, in, hi, lo);
+      hs_launch(permute_split_kernel<1, NB, T>, grid, 256, 0, s, arg, pads, in, hi, lo);
     else
-      hs_launch(permute_split_kernel<2, NB, T>, grid, 256, 0, s, arg, in, hi, lo);
+      hs_launch(permute_split_kernel<2, NB, T>, grid, 256, 0, s, arg, pads, in, hi, lo);
   };
   if (plan.nbox <= 2)
     go(std::integral_constant<int, 2>{});
@@ -565,13 +586,13 @@ cudaError_t launch_permute_split_t(const PermPlan& plan, const T* in, void* hi, 
 }
 
 cudaError_t launch_permute_split(const PermPlan& plan, const double* in, void* hi, void* lo, int mode,
-                                 cudaStream_t s) {
-  return launch_permute_split_t(plan, in, hi, lo, mode, s);
+                                 cudaStream_t s, const SplitPads& pads) {
+  return launch_permute_split_t(plan, in, hi, lo, mode, s, pads);
 }
 
 cudaError_t launch_permute_split_f32(const PermPlan& plan, const float* in, void* hi, void* lo, int mode,
-                                     cudaStream_t s) {
-  return launch_permute_split_t(plan, in, hi, lo, mode, s);
+                                     cudaStream_t s, const SplitPads& pads) {
+  return launch_permute_split_t(plan, in, hi, lo, mode, s, pads);
 }
 
 template <int MODE>
