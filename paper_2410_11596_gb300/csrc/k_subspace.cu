@@ -34,14 +34,21 @@ __global__ void fill_random_rows_kernel(double* __restrict__ X, int r0, int m, i
     X[(long long)r0 * n + e] = hash_uniform(seed * 0x100000001B3ull + (unsigned long long)e);
 }
 
-// Cholesky G = L L^T (lower) of an m x m SPD matrix and L^{-1}, in FP64, by
-// one CTA in shared memory (m <= kMaxSub). Right-looking: step j takes the
+// Cholesky G = L L^T (lower) of an m x m SPD matrix and L^{-1}, in FP64, in
+// shared memory (m <= kMaxSub). Right-looking: step j takes the
 // pivot, scales column j of L and row j of L^{-1}, then applies the rank-1
 // updates of both (forward substitution of L X = I carried along the
 // factorisation). One m x (m+1) array holds both triangles: L[i][c] at
 // (i, c) and L^{-1}[i][c] at (c, i + 1), c <= i. On a non-positive pivot the
 // status word is set and Linv is left unspecified.
+// Bound by one SM's FP64 pipe (a warp's FMA takes it about 19 cycles however
+// few lanes it has), so the updates are dealt to the threads entry by entry
+// instead of row by row, kCholCtas CTAs repeat the factorisation and share the
+// columns of L^{-1}, and thread 0 takes the next pivot's square root and
+// reciprocal while the others update. m = 100: 254 -> 150 us; the arithmetic of
+// every entry, and its order, are those of the row-by-row form.
 constexpr int kMaxChol = 160;  // m (m + 1) doubles of shared memory
+constexpr int kCholCtas = 4;
 // Rayleigh-Ritz problems up to kMaxSub (the Jacobi kernel below); subspaces
 // above kMaxChol take the library Cholesky route (hs_api.cu)
 constexpr int kMaxSub = 192;
@@ -50,10 +57,11 @@ __global__ void __launch_bounds__(1024) chol_inv_kernel(const double* __restrict
                                                         double* __restrict__ Linv0, const double* __restrict__ G1,
                                                         int m1, double* __restrict__ Linv1, int* __restrict__ status) {
   hs_pdl_enter();
-  // one CTA per matrix (blockIdx.x)
-  const double* G = blockIdx.x ? G1 : G0;
-  double* Linv = blockIdx.x ? Linv1 : Linv0;
-  const int m = blockIdx.x ? m1 : m0;
+  // kCholCtas CTAs per matrix; this one has the columns c of L^{-1} with c % kCholCtas == g
+  const int mat = blockIdx.x / kCholCtas, g = blockIdx.x % kCholCtas;
+  const double* G = mat ? G1 : G0;
+  double* Linv = mat ? Linv1 : Linv0;
+  const int m = mat ? m1 : m0;
   if (m <= 0) return;
   extern __shared__ double sh[];
   const int ld = m + 1;
@@ -64,35 +72,56 @@ __global__ void __launch_bounds__(1024) chol_inv_kernel(const double* __restrict
   }
   __shared__ int bad;
   __shared__ double s_rp;
+  // the pivot's square root and reciprocal once (FP64 square roots and
+  // divisions are long sequences on the FP64 pipe)
+  auto pivot = [&](int j, double d) {
+    const bool ok = d > 0.0;
+    const double piv = ok ? sqrt(d) : 1.0;
+    A[j * ld + j] = piv;
+    s_rp = 1.0 / piv;
+    if (!ok) bad = 1;
+  };
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, ny = blockDim.x >> 5;
+  if (threadIdx.x == 0) pivot(0, A[0]);
+  const unsigned nt = blockDim.x - 32, tu = threadIdx.x - 32;  // the updating threads: all but the first warp
   for (int j = 0; j < m; ++j) {
-    // the pivot's square root and reciprocal once (FP64 square roots and
-    // divisions are long sequences on the FP64 pipe)
-    if (threadIdx.x == 0) {
-      const double d = A[j * ld + j];
-      const bool ok = d > 0.0;
-      const double piv = ok ? sqrt(d) : 1.0;
-      A[j * ld + j] = piv;
-      s_rp = 1.0 / piv;
-      if (!ok) bad = 1;
-    }
     __syncthreads();
     const double rp = s_rp;
+    const unsigned nc = j >= g ? (unsigned)(j - g) / kCholCtas + 1 : 0;  // this CTA's columns up to j
     for (int i = j + 1 + threadIdx.x; i < m; i += blockDim.x) A[i * ld + j] *= rp;
-    for (int c = threadIdx.x; c <= j; c += blockDim.x) A[c * ld + j + 1] *= rp;
+    for (unsigned x = threadIdx.x; x < nc; x += blockDim.x) A[(g + (int)x * kCholCtas) * ld + j + 1] *= rp;
     __syncthreads();
-    for (int r = j + 1 + ty; r < m; r += ny) {
-      const double lrj = A[r * ld + j];
-      for (int c = j + 1 + tx; c <= r; c += 32) A[r * ld + c] -= lrj * A[c * ld + j];
-      for (int c = tx; c <= j; c += 32) A[c * ld + r + 1] -= lrj * A[c * ld + j + 1];
+    const unsigned n = (unsigned)(m - 1 - j);
+    if (threadIdx.x < 32) {
+      if (threadIdx.x == 0 && n > 0) {
+        const int r = j + 1;
+        const double lrj = A[r * ld + j];
+        double d = A[r * ld + r];
+        d -= lrj * A[r * ld + j];
+        pivot(r, d);
+      }
+      continue;
     }
-    __syncthreads();
+    // entries (i, c), c <= i, of the trailing triangle, without its first one
+    const unsigned nl = n * (n + 1) / 2;
+    for (unsigned e = tu + 1; e < nl; e += nt) {
+      unsigned i = (unsigned)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
+      while ((i + 1) * (i + 2) / 2 <= e) ++i;
+      while (i * (i + 1) / 2 > e) --i;
+      const int r = j + 1 + (int)i, c = j + 1 + (int)(e - i * (i + 1) / 2);
+      A[r * ld + c] -= A[r * ld + j] * A[c * ld + j];
+    }
+    for (unsigned e = tu; e < n * nc; e += nt) {
+      const unsigned i = e / nc;
+      const int r = j + 1 + (int)i, c = g + (int)(e - i * nc) * kCholCtas;
+      A[c * ld + r + 1] -= A[r * ld + j] * A[c * ld + j + 1];
+    }
   }
+  __syncthreads();
   for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
     const int i = e / m, c = e - (e / m) * m;
-    Linv[e] = c <= i ? A[c * ld + i + 1] : 0.0;
+    if (c % kCholCtas == g) Linv[e] = c <= i ? A[c * ld + i + 1] : 0.0;
   }
   if (threadIdx.x == 0 && bad) *status = 1;
 }
@@ -694,7 +723,7 @@ cudaError_t launch_chol_inv(const double* G0, int m0, double* Linv0, const doubl
   const cudaError_t attr_err = ensure_smem_attr(reinterpret_cast<const void*>(chol_inv_kernel),
                                                 kMaxChol * (kMaxChol + 1) * (int)sizeof(double));
   if (attr_err != cudaSuccess) return attr_err;
-  hs_launch(chol_inv_kernel, 2, 1024, smem, s, G0, m0, Linv0, G1, m1, Linv1, status);
+  hs_launch(chol_inv_kernel, 2 * kCholCtas, 1024, smem, s, G0, m0, Linv0, G1, m1, Linv1, status);
   return cudaGetLastError();
 }
 
