@@ -3,6 +3,7 @@
 // (Sec. II.B).
 #include <algorithm>
 #include <climits>
+#include <system_error>
 #include <utility>
 
 #include "hs_ctx.cuh"
@@ -291,6 +292,10 @@ struct Solver {
 Solver solver_of(hs_ctx ctx, int which, bool f32) {
   if (which == 0) return {ctx->solver, ctx->params, f32 ? &ctx->solver32_dev : &ctx->solver_dev,
                           f32 ? &ctx->solver32_host : &ctx->solver_host};
+  if (which >= 2) {  // FP64 only
+    hs_ctx_s::Lane& l = ctx->lane[which - 2];
+    return {l.solver, l.params, &l.dev, &l.host};
+  }
   return {ctx->solver2, ctx->params2, f32 ? &ctx->solver2_32_dev : &ctx->solver2_dev,
           f32 ? &ctx->solver2_32_host : &ctx->solver2_host};
 }
@@ -356,6 +361,64 @@ hs_status eig_pair_impl(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* 
 
 hs_status eig_pair(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, int n1, void* w1) {
   return eig_pair_impl(ctx, f32, A0, n0, w0, A1, n1, w1);
+}
+static hs_status quad_lanes(hs_ctx ctx, int nmax) {
+  int i = 2;
+  for (hs_ctx_s::Lane& l : ctx->lane) {
+    if (!l.stream) HS_CUDA(cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking));
+    if (!l.join) HS_CUDA(cudaEventCreateWithFlags(&l.join, cudaEventDisableTiming));
+    if (!l.solver) HS_SOLVER(cusolverDnCreate(&l.solver));
+    HS_SOLVER(cusolverDnSetStream(l.solver, l.stream));
+    if (!l.params) HS_SOLVER(cusolverDnCreateParams(&l.params));
+    HS_TRY(eig_ws(solver_of(ctx, i++, false), nmax, false));
+  }
+  return HS_OK;
+}
+// The blocks' Householder reductions run on one or a few SMs each, so four of
+// them side by side take little longer than two (HOTRG D = 4, chi = 32, three
+// steps: 83 -> 71 ms). Where the two more solvers and their workspaces cannot be
+// had, one pair follows the other.
+hs_status eig_quad(hs_ctx ctx, double* const A[4], int n0, int n1, double* const w[4]) {
+  const int nmax = n0 > n1 ? n0 : n1;
+  HS_TRY(eig_workspace_impl(ctx, nmax));
+  if (quad_lanes(ctx, nmax) != HS_OK) {
+    cudaGetLastError();
+    HS_TRY(eig_pair(ctx, false, A[0], n0, w[0], A[1], n1, w[1]));
+    HS_TRY(eig_pair(ctx, false, A[2], n0, w[2], A[3], n1, w[3]));
+    int* info = static_cast<int*>(ctx->info.p);
+    HS_CUDA(cudaMemcpyAsync(info + 2, info, 2 * sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
+    return HS_OK;
+  }
+  cudaStream_t side[3] = {ctx->stream2, ctx->lane[0].stream, ctx->lane[1].stream};
+  cudaEvent_t join[3] = {ctx->ev_join, ctx->lane[0].join, ctx->lane[1].join};
+  HS_CUDA(cudaEventRecord(ctx->ev_fork, ctx->stream));
+  for (cudaStream_t s : side) HS_CUDA(cudaStreamWaitEvent(s, ctx->ev_fork, 0));
+  // the solver blocks its calling thread: one thread per block
+  hs_status st[4] = {HS_OK, HS_OK, HS_OK, HS_OK};
+  std::string msg[4];
+  std::thread th[3];
+  auto solve = [&](int i) {
+    cudaSetDevice(ctx->device);
+    st[i] = eig_any(ctx, i, false, A[i], i % 2 ? n1 : n0, w[i], i);
+    if (st[i] != HS_OK) msg[i] = last_error();
+  };
+  for (int i = 1; i < 4; ++i) {
+    try {
+      th[i - 1] = std::thread(solve, i);
+    } catch (const std::system_error&) {  // no thread to be had
+      solve(i);
+    }
+  }
+  solve(0);
+  for (std::thread& t : th)
+    if (t.joinable()) t.join();
+  for (int i = 0; i < 3; ++i) {
+    HS_CUDA(cudaEventRecord(join[i], side[i]));
+    HS_CUDA(cudaStreamWaitEvent(ctx->stream, join[i], 0));
+  }
+  for (int i = 0; i < 4; ++i)
+    if (st[i] != HS_OK) return fail(st[i], "%s", msg[i].c_str());
+  return HS_OK;
 }
 hs_status eig_single(hs_ctx ctx, bool f32, void* A, int n, void* w) { return eig_any(ctx, 0, f32, A, n, w, 0); }
 hs_status eig_workspace32(hs_ctx ctx, int nmax) { return eig32_workspace(ctx, nmax); }
@@ -1675,6 +1738,14 @@ hs_status hs_destroy(hs_ctx ctx) {
   if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
   if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
   if (ctx->stream2) cudaStreamDestroy(ctx->stream2);
+  for (hs_ctx_s::Lane& l : ctx->lane) {
+    if (l.stream) cudaStreamSynchronize(l.stream);
+    l.dev.release();
+    if (l.params) cusolverDnDestroyParams(l.params);
+    if (l.solver) cusolverDnDestroy(l.solver);
+    if (l.join) cudaEventDestroy(l.join);
+    if (l.stream) cudaStreamDestroy(l.stream);
+  }
   if (ctx->params) cusolverDnDestroyParams(ctx->params);
   if (ctx->solver) cusolverDnDestroy(ctx->solver);
   if (ctx->blas) cublasDestroy(ctx->blas);

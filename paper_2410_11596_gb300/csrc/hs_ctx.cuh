@@ -158,6 +158,16 @@ struct hs_ctx_s {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   hs::DBuf solver2_dev, solver2_32_dev;
   std::vector<char> solver2_host, solver2_32_host;
+  // two more solvers, made by the first HOTRG step: the two Gram matrices' four
+  // blocks are diagonalised at once (eig_quad)
+  struct Lane {
+    cudaStream_t stream = nullptr;
+    cusolverDnHandle_t solver = nullptr;
+    cusolverDnParams_t params = nullptr;
+    cudaEvent_t join = nullptr;
+    hs::DBuf dev;
+    std::vector<char> host;
+  } lane[2];
   // HOTRG workspace
   hs::DBuf hb[16];
   // complex (graded) CTMRG: private copy of a~ followed by its conjugate, and scratch
@@ -275,6 +285,9 @@ hs_status permute(hs_ctx ctx, const Z2Mat& in, const Z2Mat& out, std::initialize
 // stream); FP32 when f32. Shared with the HOTRG step.
 hs_status eig_pair(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, int n1, void* w1);
 hs_status eig_workspace(hs_ctx ctx, int nmax);
+// Two pairs of blocks (n0 and n1 each) at once, FP64: A[0], A[1] with eigenvalues
+// w[0], w[1], then A[2], A[3]; the second pair's info in ctx->info[2..3].
+hs_status eig_quad(hs_ctx ctx, double* const A[4], int n0, int n1, double* const w[4]);
 // One symmetric eigen-decomposition (vectors in place, column-major) on the
 // context stream; FP32 when f32 (workspace from eig_workspace32).
 hs_status eig_single(hs_ctx ctx, bool f32, void* A, int n, void* w);
