@@ -296,6 +296,56 @@ HS_HD bool f32_widen_fast(uint32_t f, unsigned long long& out) {
   return true;
 }
 
+// x[0] + x[1] + ... + x[n - 1] added one after the other in FP64 (n <= MAX <= 16).
+// With exponents within 25 of the largest every x is a multiple of
+// u = 2^(emax - 175) and all partial sums stay below 2^53 u, so that every FP64
+// add is exact and the sum can be taken in integers, off the FP64 pipe. A wider
+// spread, subnormals, infinities and NaN take the adds.
+template <int MAX>
+HS_HD double sum_f32_in_f64(const float (&x)[MAX], int n) {
+  static_assert(MAX <= 16, "2^4 * 2^24 * 2^25 = 2^53");
+  uint32_t u[MAX], top = 0u, low = 0x7F800000u;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int s = 0; s < MAX; ++s) {
+    if (s >= n) break;
+    std::memcpy(&u[s], &x[s], 4);
+    const uint32_t mag = u[s] & 0x7FFFFFFFu;
+    top = top > mag ? top : mag;
+    low = mag != 0u && mag < low ? mag : low;
+  }
+  const int emax = (int)(top >> 23);
+  if (emax < 255 && low >= 0x00800000u && emax - (int)(low >> 23) <= 25) {
+    long long v = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int s = 0; s < MAX; ++s) {
+      if (s >= n) break;
+      const uint32_t e = (u[s] >> 23) & 0xFFu;
+      const int m = e ? (int)((u[s] & 0x7FFFFFu) | 0x800000u) : 0;
+      v += (long long)((u[s] >> 31) ? -m : m) * (1 << ((e + 25u - (uint32_t)emax) & 31u));
+    }
+    if (v == 0) return 0.0;
+    const unsigned long long a = (unsigned long long)(v < 0 ? -v : v);
+    const int z = clz64(a);
+    const unsigned long long ex = (unsigned long long)(1023 + 63 - z + emax - 175);
+    return f64_from_bits((v < 0 ? 1ull << 63 : 0ull) | (ex << 52) | ((a << (z - 11)) & ((1ull << 52) - 1)));
+  }
+  double v = 0.0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int s = 0; s < MAX; ++s) {
+    if (s >= n) break;
+    unsigned long long w;
+    if (!f32_widen_fast(u[s], w)) w = f64_bits((double)x[s]);  // subnormal
+    v += f64_from_bits(w);
+  }
+  return v;
+}
+
 // ---- FP64 operands as slices of 8-bit digits (k_gemm_sl.cu) -------------------
 //
 // A row whose largest biased exponent field is emax is written as

@@ -589,26 +589,47 @@ struct SplitRed {
 struct SplitReds {
   SplitRed r[kMaxPairs];
 };
+constexpr int kRedThreads = 128;
+constexpr int kMaxSplits = 16;  // sum_f32_in_f64's limit
 
-__global__ void tc_splitk_reduce_kernel(const SplitReds reds) {
+// A chain of FP64 adds is bound by the FP64 pipe (8 partials of 96 x 2592 on two
+// blocks: 4 M adds at 260 a cycle are 8 us, the partials' 16 MB 3 us), hence the
+// integer sum of hs_bits.cuh: 7.5 -> 4.9 us a launch on average over the
+// subspace steps at n = 2592, same bits. Two columns a thread: 8-byte loads.
+__global__ void __launch_bounds__(kRedThreads) tc_splitk_reduce_kernel(const SplitReds reds) {
   hs_pdl_enter();
   const SplitRed& r = reds.r[blockIdx.y];
-  const long long mn = (long long)r.M * r.N, stride = (long long)r.M * r.ldp;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < mn;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long row = e / r.N, col = e - row * r.N;
-    double v = 0.0;
-    for (int s = 0; s < r.nsplit; ++s) {
-      // widened on the bit pattern (the FP64 pipe, which a conversion would use, is GB300's scarce one)
-      const uint32_t x = __float_as_uint(r.part[s * stride + row * r.ldp + col]);
-      unsigned long long w;
-      if (!f32_widen_fast(x, w)) w = f64_bits((double)__uint_as_float(x));  // subnormal
-      v += f64_from_bits(w);
+  const unsigned half = (unsigned)r.ldp / 2;
+  const long long pairs = (long long)r.M * half, stride = (long long)r.M * half;
+  const float2* part = reinterpret_cast<const float2*>(r.part);
+  for (long long e = (long long)blockIdx.x * kRedThreads + threadIdx.x; e < pairs;
+       e += (long long)gridDim.x * kRedThreads) {
+    // 32-bit division where the index allows it
+    const long long row = pairs < (1ll << 32) ? (long long)((unsigned)e / half) : e / half;
+    const int col = 2 * (int)(e - row * half);
+    float x0[kMaxSplits], x1[kMaxSplits];
+#pragma unroll
+    for (int s = 0; s < kMaxSplits; ++s) {
+      if (s >= r.nsplit) break;
+      const float2 t = part[s * stride + e];
+      x0[s] = t.x;
+      x1[s] = t.y;
     }
-    if (r.f32)
-      reinterpret_cast<float*>(r.c)[row * r.ldc + col] = (float)v;
-    else
-      r.c[row * r.ldc + col] = v;
+    const bool two = col + 1 < r.N;  // the last column of an odd row has no partner
+    const double v0 = sum_f32_in_f64<kMaxSplits>(x0, r.nsplit), v1 = two ? sum_f32_in_f64<kMaxSplits>(x1, r.nsplit) : 0.0;
+    if (r.f32) {
+      float* c = reinterpret_cast<float*>(r.c) + row * r.ldc + col;
+      c[0] = (float)v0;
+      if (two) c[1] = (float)v1;
+    } else {
+      double* c = r.c + row * r.ldc + col;
+      if (two && (reinterpret_cast<uintptr_t>(c) & 15) == 0) {
+        *reinterpret_cast<double2*>(c) = make_double2(v0, v1);
+      } else {
+        c[0] = v0;
+        if (two) c[1] = v1;
+      }
+    }
   }
 }
 
@@ -676,7 +697,7 @@ cudaError_t run(const TcProblem* probs, int nprob, int* err, cudaStream_t s, dou
     if (part && ptiles < sms && psi < 0) {
       ns = (sms + ptiles - 1) / ptiles;
       ns = ns < ktiles / 4 ? ns : ktiles / 4;
-      ns = ns < 16 ? ns : 16;
+      ns = ns < kMaxSplits ? ns : kMaxSplits;
       const long long need = (long long)ns * p.M * ((p.N + 1) & ~1);
       if (ns < 2 || part_used + need > part_felems || g.n + ns > kMaxUnits) ns = 1;
     }
@@ -728,10 +749,10 @@ cudaError_t run(const TcProblem* probs, int nprob, int* err, cudaStream_t s, dou
   if (e != cudaSuccess) return e;
   if (nred > 0) {
     long long mn = 0;
-    for (int r = 0; r < nred; ++r) mn = std::max(mn, (long long)red[r].M * red[r].N);
-    long long gx = (mn + 255) / 256;
-    if (gx > 4096) gx = 4096;
-    hs_launch(tc_splitk_reduce_kernel, dim3((unsigned)gx, (unsigned)nred), 256, 0, s, reds);
+    for (int r = 0; r < nred; ++r) mn = std::max(mn, (long long)red[r].M * (red[r].ldp / 2));
+    long long gx = (mn + kRedThreads - 1) / kRedThreads;
+    if (gx > 8192) gx = 8192;
+    hs_launch(tc_splitk_reduce_kernel, dim3((unsigned)gx, (unsigned)nred), kRedThreads, 0, s, reds);
   }
   return cudaGetLastError();
 }
