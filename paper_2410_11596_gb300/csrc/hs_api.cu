@@ -2365,8 +2365,9 @@ hs_status hs_gemm(hs_ctx ctx, hs_precision precision, int M, int N, int K, const
   HS_TRY(ctx->tc_b_hi.ensure((size_t)N * Kp * eb));
   HS_TRY(ctx->tc_b_lo.ensure((size_t)N * Kp * eb));
   ctx->tc_x_hi.zkey = ctx->tc_x_lo.zkey = ctx->tc_b_hi.zkey = ctx->tc_b_lo.zkey = 0;
-  HS_CUDA(launch_split_pad(A, M, K, lda, ctx->tc_x_hi.p, ctx->tc_x_lo.p, Kp, tc_mode(precision), ctx->stream));
-  HS_CUDA(launch_split_pad(B, N, K, ldb, ctx->tc_b_hi.p, ctx->tc_b_lo.p, Kp, tc_mode(precision), ctx->stream));
+  const SplitPadOp ops[2] = {{A, M, K, lda, ctx->tc_x_hi.p, ctx->tc_x_lo.p, Kp},
+                             {B, N, K, ldb, ctx->tc_b_hi.p, ctx->tc_b_lo.p, Kp}};
+  HS_CUDA(launch_split_pads(ops, 2, tc_mode(precision), ctx->stream));
   TcProblem t;
   t.M = M;
   t.N = N;

@@ -82,12 +82,13 @@ hs_status ggemm(hs_ctx ctx, hs_precision prec, const GMat& Am, const double* A, 
   ctx->sx_hi.zkey = ctx->sx_lo.zkey = ctx->sy_hi.zkey = ctx->sy_lo.zkey = 0;
   {
     PhaseScope ps(ctx, HS_PHASE_PERMUTE);
-    HS_CUDA(launch_split_pad(A, ra, (int)K, g_ld(Am), ctx->sx_hi.p, ctx->sx_lo.p, Kp, mode, ctx->stream));
     // B~ and its conjugate (stored g_elems(Bm) apart) split back to back
-    HS_CUDA(launch_split_pad(B, rb, (int)K, g_ld(Bm), ctx->sy_hi.p, ctx->sy_lo.p, Kp, mode, ctx->stream));
-    HS_CUDA(launch_split_pad(B + g_elems(Bm), rb, (int)K, g_ld(Bm), static_cast<char*>(ctx->sy_hi.p) + rb * Kp * eb,
-                             static_cast<char*>(ctx->sy_lo.p) + rb * Kp * eb, Kp, mode, ctx->stream));
-    ctx->launches += 3;
+    const SplitPadOp ops[3] = {{A, ra, (int)K, g_ld(Am), ctx->sx_hi.p, ctx->sx_lo.p, Kp},
+                               {B, rb, (int)K, g_ld(Bm), ctx->sy_hi.p, ctx->sy_lo.p, Kp},
+                               {B + g_elems(Bm), rb, (int)K, g_ld(Bm), static_cast<char*>(ctx->sy_hi.p) + rb * Kp * eb,
+                                static_cast<char*>(ctx->sy_lo.p) + rb * Kp * eb, Kp}};
+    HS_CUDA(launch_split_pads(ops, 3, mode, ctx->stream));
+    ctx->launches += 1;
   }
   TcProblem pr[4];
   int np = 0;

@@ -341,10 +341,19 @@ cudaError_t launch_join_split_f32(const void* hi, const void* lo, long long rows
 cudaError_t launch_permute_split(const PermPlan& plan, const double* in, void* hi, void* lo, int mode,
                                  cudaStream_t s, const SplitPads& pads = SplitPads());
 
-// Split a row-major FP64 matrix [rows, cols] (row stride ld_src) into padded
-// hi/lo operands [rows, ld_dst] (zeros in columns cols..ld_dst-1); mode as above.
-cudaError_t launch_split_pad(const double* src, long long rows, int cols, long long ld_src, void* hi,
-                             void* lo, long long ld_dst, int mode, cudaStream_t s);
+// A row-major FP64 matrix [rows, cols] (row stride ld_src) to be split into padded
+// hi/lo operands [rows, ld_dst] (zeros in columns cols..ld_dst-1; 16-byte aligned,
+// ld_dst a multiple of 4), and up to three of them in one launch; mode as above.
+struct SplitPadOp {
+  const double* src;
+  long long rows;
+  int cols;
+  long long ld_src;
+  void *hi, *lo;
+  long long ld_dst;
+};
+constexpr int kMaxSplitPads = 3;
+cudaError_t launch_split_pads(const SplitPadOp* ops, int n, int mode, cudaStream_t s);
 
 // ---- tensor-core (tcgen05) block GEMM ------------------------------------------
 

@@ -89,8 +89,8 @@ extern "C" hs_status hs_gemm_static(hs_precision precision, int M, int N, int K,
   unsigned char* b_hi = a_lo + (size_t)M * Kp * eb;
   unsigned char* b_lo = b_hi + (size_t)N * Kp * eb;
   const int mode = tc_mode(precision);
-  HS_CUDA(launch_split_pad(A, M, K, lda, a_hi, a_lo, Kp, mode, s));
-  HS_CUDA(launch_split_pad(B, N, K, ldb, b_hi, b_lo, Kp, mode, s));
+  const SplitPadOp ops[2] = {{A, M, K, lda, a_hi, a_lo, Kp}, {B, N, K, ldb, b_hi, b_lo, Kp}};
+  HS_CUDA(launch_split_pads(ops, 2, mode, s));
   TcProblem t;
   t.M = M;
   t.N = N;
