@@ -44,12 +44,12 @@ FLUSH_BYTES = 512 << 20
 # DRAM traffic per launch of the roofline kernel from one ncu capture, valid only
 # while the kernel source is unchanged (sha256 of the file, first 16 hex digits).
 NCU_TRAFFIC = {
-    # FP64 block GEMM, one ncu capture of a D=6 chi=144 move: mean of its G3/G4/G5 launches
-    "gemm_f64": {"bytes_per_launch": 143.3e6, "source_sha": "ac07f1d8a4d24d63"},
+    # FP64 block GEMM by digit slices, one ncu capture of a 10368 x 666 x 666 product: its operand split and GEMM
+    "gemm_sl": {"bytes_per_launch": 239.4e6, "source_sha": "a70f7fc166e94f07"},
     # tensor-core GEMM, one ncu capture of two steady-state D=6 chi=144 moves: mean over its launches
-    "gemm_tc_tf32x3": {"bytes_per_launch": 56.6e6, "source_sha": "c3b7279478e6ad5a"},
+    "gemm_tc_tf32x3": {"bytes_per_launch": 56.5e6, "source_sha": "751d5096e63fff00"},
     # the same capture, mean over its split-output launches (G2-G5, the dominant kernel)
-    "gemm_tc_split_tf32x3": {"bytes_per_launch": 131.5e6, "source_sha": "c3b7279478e6ad5a"},
+    "gemm_tc_split_tf32x3": {"bytes_per_launch": 131.3e6, "source_sha": "751d5096e63fff00"},
 }
 
 EIG_LABEL = {"f64": "FP64 syevd per parity block", "f32p": "FP32 syevd + FP64 Loewdin and projection",
@@ -261,21 +261,6 @@ class Clocks:
         reasons = sorted({names[i] for _, _, r in rows for i, v in enumerate(r) if v.lower() == "active"})
         return {"sm_mhz": float(np.median([r[0] for r in rows])), "sm_max_mhz": max(r[1] for r in rows),
                 "reasons": reasons, "samples": len(rows)}
-
-
-def fp64_peak_tflops(torch, dev):
-    """cuBLAS DGEMM 4096^3, best of 4 (the FP64 pipe's measured rate on this GPU)."""
-    a = torch.randn(4096, 4096, dtype=torch.float64, device=dev)
-    b = torch.randn(4096, 4096, dtype=torch.float64, device=dev)
-    best = 1e9
-    for _ in range(4):
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record()
-        a @ b
-        e1.record()
-        e1.synchronize()
-        best = min(best, e0.elapsed_time(e1))
-    return 2 * 4096 ** 3 / (best * 1e-3) / 1e12
 
 
 def measured_bf16_tflops():
@@ -655,9 +640,11 @@ def run_ours(args):
     total_ms = float(np.sum(ms_r))
     if args.precision == "f64":
         k_ms, k_flops = prof_r["phase_ms"]["gemm"], prof_r["phase_flops"]["gemm"]
-        src, key = "paper_2410_11596_gb300/csrc/k_gemm_f64.cu", "gemm_f64"
-        peak, bound, kname = fp64_peak_tflops(torch, dev), "alu", "gemm_f64_nt_kernel (Z2 block GEMM, DFMA)"
-        psrc = "FP64: cuBLAS DGEMM 4096^3 measured in this run"
+        src, key = "paper_2410_11596_gb300/csrc/k_gemm_sl.cu", "gemm_sl"
+        bf16, how = measured_bf16_tflops()
+        peak, bound = bf16 / 34, "tensor"
+        kname = "gemm_sl_kernel and its operand splits (Z2 block GEMM, 34 BF16 products of 8-bit digit slices)"
+        psrc = f"bf16 burst {bf16:.1f} TF/s (of {how}) / 34 digit products per FP64 product"
     else:
         # the dominant kernel: the split-output instantiation of the tcgen05 GEMM (the enlarged corner
         # and edge products G2-G5, 35% of a steady-state move's kernel time in the ncu launch list);

@@ -17,7 +17,7 @@
 // entries. Joining the third edge to the ring first and contracting the open
 // double layer as one q^3 index took 2 c^3 q^3 + 2 c^2 d^2 q^4 operations and
 // two arrays of c^2 q^3 (D = 6, c = 144: 836 against 94 GFLOP for both sites,
-// 15.5 against 2.6 GB). eps joins two half rings over both of their boundary
+// 15.5 against 2.6 GB; 231 -> 10.5 ms with the same GEMM kernels). eps joins two half rings over both of their boundary
 // bonds, 4 c^3 q^2 + 2 c^2 q^4 operations instead of 2 c^3 q^3 + 2 c^2 q^4.
 #include "hs_ctx.cuh"
 
@@ -314,8 +314,8 @@ __global__ void finish_rho_c_kernel(const double* __restrict__ re4, const double
 constexpr int kRhoParts = 64;
 
 // Partial sums of rho4[s1, s1', s2, s2'] = sum_{x0, mk, mb, x4} L R: part[pair][i]
-// from every kRhoParts-th (x0, mk, mb). Bound by the FP64 pipe (d^4 c^2 q FMAs,
-// 23 us at D = 6, c = 144), with the operands read from L2; a 4 x 4 GEMM over
+// from every kRhoParts-th (x0, mk, mb). The d^4 c^2 q FMAs are 23 us of the FP64
+// pipe at D = 6, c = 144; it takes 161 us, waiting for its operands from L2; a 4 x 4 GEMM over
 // c^2 q would leave 255 of 256 tile entries idle.
 __global__ void __launch_bounds__(128) rho4_kernel(const double* __restrict__ Lr, const double* __restrict__ Li,
                                                    const double* __restrict__ Rr, const double* __restrict__ Ri, int d,

@@ -158,7 +158,7 @@ __global__ void double_layer_graded_kernel(const double* __restrict__ A, int d, 
 
 // One warp per row (x_u, x_l, x_d) of q contiguous entries: the row's ket and
 // bra offsets into A once, 32-bit indices inside. Bound by the FP64 pipe (d FMAs
-// per entry) and the write.
+// per entry) and the write: 47 -> 33 us at D = 7.
 __global__ void __launch_bounds__(256) double_layer_dense_kernel(const double* __restrict__ A, int d, int D, bool cplx,
                                                                  double* __restrict__ out) {
   hs_pdl_enter();
@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(256) double_layer_dense_kernel(const double* _
 // the 16 rotated ones by four rounds of sums and differences. One thread per
 // four leg classes P (P < D: the state (P P'), else pair P - D): every plain
 // entry is read once, 4 additions an entry (16 gathered reads and 16 FMAs of a
-// product of four coefficients before: 1354 us at D = 7, now bound by the FP64
-// pipe). Lanes run over the last leg, whose row of q entries they share.
+// product of four coefficients before: 1354 us at D = 7, now 103 us, bound by the
+// FP64 pipe). Lanes run over the last leg, whose row of q entries they share.
 __global__ void __launch_bounds__(256) rotate_dense_kernel(const double* __restrict__ a, int D, double* __restrict__ out,
                                                            unsigned long long* maxes) {
   hs_pdl_enter();
