@@ -115,37 +115,57 @@ hs_status gemm_sliced(hs_ctx ctx, const SlMat* mats, int nm, const SlProblem* pr
                       bool accumulate, bool* done) {
   *done = false;
   if (np < 1 || ctx->no_slices || !slices_pay(probs, mats, np) || capturing(ctx->stream)) return HS_OK;
-  size_t all = 0;
-  for (int i = 0; i < nm; ++i) all += slices_bytes(mats[i].rows, mats[i].kseg * mats[i].nseg, mats[i].is_b);
+  SlMat m[2 * kMaxProblems];
+  size_t scales = 0, all = 0;
+  for (int i = 0; i < nm; ++i) {
+    const int K = mats[i].kseg * mats[i].nseg;
+    m[i] = mats[i];
+    scales += slices_scale_bytes(K);
+    all += slices_bytes(m[i].rows, K, m[i].is_b);
+  }
+  for (int i = 0; i < np; ++i) all += slices_list_bytes(m[probs[i].a].rows, m[probs[i].b].rows);
+  all += scales;
   if (ctx->sl_ws.ensure(all < kSliceBytes ? all : kSliceBytes) != HS_OK) return HS_OK;  // no memory left
   int* err = static_cast<int*>(ctx->tc_err.p);
+  char* const ws = static_cast<char*>(ctx->sl_ws.p) + scales;
+  const size_t room = ctx->sl_ws.bytes - scales;
+  HS_CUDA(launch_slice_scales(m, nm, probs, np, ctx->sl_ws.p, ctx->stream));
+  ctx->launches += 1;
+  *done = true;
   if (all <= ctx->sl_ws.bytes) {
-    HS_CUDA(launch_gemm_slices(mats, nm, probs, np, accumulate, ctx->sl_ws.p, ctx->sl_ws.bytes, err,
-                               ctx->stream));
-    ctx->launches += 2;
-    *done = true;
+    HS_CUDA(launch_gemm_slices(m, nm, probs, np, accumulate, ws, room, err, ctx->stream));
+    ctx->launches += 4;
     return HS_OK;
   }
-  const size_t half = ctx->sl_ws.bytes / 2;
   for (int i = 0; i < np; ++i) {
-    const SlMat &a = mats[probs[i].a], &b = mats[probs[i].b];
-    auto panel = [&](const SlMat& m) {
-      const int block = slices_block(m.is_b);
-      const long long r = (long long)(half / slices_bytes(block, m.kseg * m.nseg, m.is_b)) * block;
-      return (int)(r < m.rows ? r : m.rows);
+    const SlMat &a = m[probs[i].a], &b = m[probs[i].b];
+    // the smaller operand in one panel if that takes no more than 3/8 of the room, the
+    // other in what is left of 3/4; the list of a panel's entries in the last quarter
+    auto rows = [](const SlMat& x, size_t bytes) {
+      const int block = slices_block(x.is_b);
+      const long long r = (long long)(bytes / slices_bytes(block, x.kseg * x.nseg, x.is_b)) * block;
+      return (int)(r < x.rows ? r : x.rows);
     };
-    const int ra = panel(a), rb = panel(b);
+    auto size = [](const SlMat& x, int r) { return slices_bytes(r, x.kseg * x.nseg, x.is_b); };
+    int ra = rows(a, room / 8 * 3), rb = rows(b, room / 8 * 3);
+    if (rb == b.rows)
+      ra = rows(a, room / 4 * 3 - size(b, rb));
+    else if (ra == a.rows)
+      rb = rows(b, room / 4 * 3 - size(a, ra));
+    // whole waves of tiles
+    const int ba = slices_block(false), tn = (rb + slices_block(true) - 1) / slices_block(true);
+    const int sms = device_sms(), waves = (ra / ba) * tn / sms;
+    if (ra < a.rows && tn <= sms && waves > 0) ra = waves * sms / tn * ba;
+    while (ra > ba && slices_list_bytes(ra, rb) > room / 4) ra = std::max(ba, ra / 2 / ba * ba);
     if (ra < 1 || rb < 1) return fail(HS_ERR_SHAPE, "contraction of %d too long for the slices", a.kseg * a.nseg);
     for (int n0 = 0; n0 < b.rows; n0 += rb)
       for (int m0 = 0; m0 < a.rows; m0 += ra) {
         const SlMat part[2] = {row_panel(a, m0, std::min(ra, a.rows - m0)), row_panel(b, n0, std::min(rb, b.rows - n0))};
         const SlProblem pr = {0, 1, probs[i].c + (long long)m0 * probs[i].ldc + n0, probs[i].ldc};
-        HS_CUDA(launch_gemm_slices(part, 2, &pr, 1, accumulate, ctx->sl_ws.p, ctx->sl_ws.bytes, err,
-                                   ctx->stream));
-        ctx->launches += 2;
+        HS_CUDA(launch_gemm_slices(part, 2, &pr, 1, accumulate, ws, room, err, ctx->stream));
+        ctx->launches += 4;
       }
   }
-  *done = true;
   return HS_OK;
 }
 }  // namespace

@@ -47,6 +47,16 @@ HS_HD double f64_from_bits(unsigned long long b) {
 #endif
 }
 
+HS_HD float f32_from_bits(uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float x;
+  std::memcpy(&x, &b, 4);
+  return x;
+#endif
+}
+
 // Quotient n / d for 32-bit n from magic numbers of d (Granlund and
 // Montgomery, PLDI 1994, unsigned division by invariant integers):
 // l = ceil(log2 d), mag = floor(2^32 (2^l - d) / d) + 1, sh1 = min(l, 1),
@@ -372,6 +382,34 @@ HS_HD long long slice_bias(long long X) { return X + 0x808080808080ll; }
 // Digit d_i (i = 1..7) of the biased value.
 HS_HD int slice_digit(long long Y, int i) {
   return i == 1 ? (int)(Y >> 48) : (int)((unsigned long long)Y >> (8 * (7 - i)) & 0xFF) - 128;
+}
+
+// x 2^adj of the double with bits b (|adj| < 1024): zeros, subnormals, infinities and
+// NaN as they are, what overflows an infinity, what underflows the smallest subnormal.
+HS_HD unsigned long long slice_scaled(unsigned long long b, int adj) {
+  const int ef = (int)((b >> 52) & 0x7FF), e2 = ef + adj;
+  if (ef == 0 || ef == 0x7FF) return b;
+  const unsigned long long sign = b & (1ull << 63);
+  if (e2 >= 0x7FF) return sign | 0x7FF0000000000000ull;
+  if (e2 <= 0) return sign | 1ull;
+  return sign | ((unsigned long long)e2 << 52) | (b & 0xFFFFFFFFFFFFFull);
+}
+
+// |x| of the double with bits b, as E5M2 times 2^-15 of the row's scale 2^(emax -
+// 1022): truncated to two mantissa bits, and every nonzero below 2^-29 of the scale
+// raised to that, so that products of two such bytes sum to zero only if all terms
+// are zero.
+HS_HD uint32_t slice_mag8(unsigned long long b, int emax) {
+  const unsigned long long mag = b & 0x7FFFFFFFFFFFFFFFull;
+  const int v = (int)(mag >> 50) - (emax - 29) * 4;
+  return mag == 0 ? 0u : (uint32_t)(v < 4 ? 4 : v);
+}
+
+// |x| over the row's scale as a float (truncated to 20 mantissa bits; zeros and
+// subnormals give less than 2^-100).
+HS_HD float slice_magf(unsigned long long b, int emax) {
+  const int t = (int)((b >> 32) & 0x7FFFFFFFu) - (emax - 126) * (1 << 20);
+  return f32_from_bits(t < 0 ? 0u : (uint32_t)t << 3);
 }
 
 // Bit pattern of the double J 2^s, |J| < 2^63, rounded to nearest even; 0 for

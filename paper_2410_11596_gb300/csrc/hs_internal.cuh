@@ -413,6 +413,7 @@ struct SlMat {
   int nseg, kseg, rows;
   long long ld;
   bool is_b;  // an N-side operand (its digit planes are laid out in other row blocks)
+  const short* scale = nullptr;  // scales of the columns (launch_slice_scales)
 };
 // C[rows of mats[a], rows of mats[b]] = A B^T (+ C).
 struct SlProblem {
@@ -420,11 +421,18 @@ struct SlProblem {
   double* c;
   int ldc;
 };
-// Workspace bytes of one operand (rows in whole blocks when it is a panel); whether the slices beat the FP64 kernel.
+// Workspace bytes of one operand (rows in whole blocks when it is a panel), of its
+// columns' scales and of the list of an M x N product's entries that are summed again; whether the slices beat the FP64 kernel.
 size_t slices_bytes(int rows, int K, bool is_b);
+size_t slices_scale_bytes(int K);
+size_t slices_list_bytes(long long M, long long N);
 int slices_block(bool is_b);  // rows per block of the planes
 bool slices_pay(const SlProblem* probs, const SlMat* mats, int n);
-// Up to 8 operands and 4 problems per call (K <= 65536); err as for launch_gemm_tc.
+// Fills the operands' scales, in ws (their slices_scale_bytes), for a following launch_gemm_slices of
+// them or of panels of their rows.
+cudaError_t launch_slice_scales(SlMat* mats, int nmat, const SlProblem* probs, int nprob, void* ws, cudaStream_t s);
+// Up to 8 operands and 4 problems per call (K <= 65536); err as for launch_gemm_tc. ws holds the
+// operands' slices and the problems' lists.
 cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob,
                                bool accumulate, void* ws, size_t ws_bytes, int* err, cudaStream_t s);
 
