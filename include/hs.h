@@ -422,7 +422,8 @@ hs_status hs_hotrg_init(hs_ctx ctx, const hs_z2_tensor* a, hs_z2_tensor* t, doub
  * stacking). The isometry is the top-chi eigenvector set of the left or the
  * right Gram matrix of the fused leg, whichever discards less weight (ties:
  * left); one FP64 eigen-decomposition per parity block, states kept across
- * both blocks by eigenvalue. The new tensor is divided by its largest
+ * both blocks by eigenvalue. A side one of whose decompositions fails is not
+ * taken; HS_ERR_SOLVER if both fail. The new tensor is divided by its largest
  * modulus. precision: HS_PREC_F64 runs the block GEMMs on the FP64 kernel;
  * HS_PREC_TF32X3 / TF32 / BF16X3 run them on tcgen05 (operands split straight
  * from their source layouts, FP32 accumulation, FP64 output); the Gram

@@ -354,10 +354,11 @@ hs_status eig_any(hs_ctx ctx, int which, bool f32, void* A, int n, void* w, int 
 
 // Both parity blocks: block 0 on the context stream, block 1 on the second
 // stream from a helper thread (cuSOLVER's syevd blocks its calling thread).
-hs_status eig_pair_impl(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, int n1, void* w1) {
+// Their statuses go to info[slot], info[slot + 1].
+hs_status eig_pair_impl(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, int n1, void* w1, int slot) {
   if (n0 == 0 || n1 == 0) {
-    HS_TRY(eig_any(ctx, 0, f32, A0, n0, w0, 0));
-    return eig_any(ctx, 0, f32, A1, n1, w1, 1);
+    HS_TRY(eig_any(ctx, 0, f32, A0, n0, w0, slot));
+    return eig_any(ctx, 0, f32, A1, n1, w1, slot + 1);
   }
   HS_CUDA(cudaEventRecord(ctx->ev_fork, ctx->stream));
   HS_CUDA(cudaStreamWaitEvent(ctx->stream2, ctx->ev_fork, 0));
@@ -365,10 +366,10 @@ hs_status eig_pair_impl(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* 
   std::string err1;
   std::thread th([&] {
     cudaSetDevice(ctx->device);
-    st1 = eig_any(ctx, 1, f32, A1, n1, w1, 1);
+    st1 = eig_any(ctx, 1, f32, A1, n1, w1, slot + 1);
     if (st1 != HS_OK) err1 = last_error();
   });
-  const hs_status st0 = eig_any(ctx, 0, f32, A0, n0, w0, 0);
+  const hs_status st0 = eig_any(ctx, 0, f32, A0, n0, w0, slot);
   th.join();
   HS_CUDA(cudaEventRecord(ctx->ev_join, ctx->stream2));
   HS_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0));
@@ -380,7 +381,7 @@ hs_status eig_pair_impl(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* 
 }  // namespace
 
 hs_status eig_pair(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, int n1, void* w1) {
-  return eig_pair_impl(ctx, f32, A0, n0, w0, A1, n1, w1);
+  return eig_pair_impl(ctx, f32, A0, n0, w0, A1, n1, w1, 0);
 }
 static hs_status quad_lanes(hs_ctx ctx, int nmax) {
   int i = 2;
@@ -403,11 +404,8 @@ hs_status eig_quad(hs_ctx ctx, double* const A[4], int n0, int n1, double* const
   HS_TRY(eig_workspace_impl(ctx, nmax));
   if (quad_lanes(ctx, nmax) != HS_OK) {
     cudaGetLastError();
-    HS_TRY(eig_pair(ctx, false, A[0], n0, w[0], A[1], n1, w[1]));
-    HS_TRY(eig_pair(ctx, false, A[2], n0, w[2], A[3], n1, w[3]));
-    int* info = static_cast<int*>(ctx->info.p);
-    HS_CUDA(cudaMemcpyAsync(info + 2, info, 2 * sizeof(int), cudaMemcpyDeviceToDevice, ctx->stream));
-    return HS_OK;
+    HS_TRY(eig_pair_impl(ctx, false, A[0], n0, w[0], A[1], n1, w[1], 0));
+    return eig_pair_impl(ctx, false, A[2], n0, w[2], A[3], n1, w[3], 2);
   }
   cudaStream_t side[3] = {ctx->stream2, ctx->lane[0].stream, ctx->lane[1].stream};
   cudaEvent_t join[3] = {ctx->ev_join, ctx->lane[0].join, ctx->lane[1].join};

@@ -286,7 +286,7 @@ hs_status permute(hs_ctx ctx, const Z2Mat& in, const Z2Mat& out, std::initialize
 hs_status eig_pair(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, int n1, void* w1);
 hs_status eig_workspace(hs_ctx ctx, int nmax);
 // Two pairs of blocks (n0 and n1 each) at once, FP64: A[0], A[1] with eigenvalues
-// w[0], w[1], then A[2], A[3]; the second pair's info in ctx->info[2..3].
+// w[0], w[1], then A[2], A[3]; their statuses in ctx->info[0..3].
 hs_status eig_quad(hs_ctx ctx, double* const A[4], int n0, int n1, double* const w[4]);
 // One symmetric eigen-decomposition (vectors in place, column-major) on the
 // context stream; FP32 when f32 (workspace from eig_workspace32).

@@ -15,6 +15,7 @@
 // The right Gram matrix is the same on the mirrored tensor (l <-> r). The
 // new tensor is T'[u, L, d, R] = sum U[(l1 l2), L] M[...] U[(r1 r2), R].
 #include "hs_ctx.cuh"
+#include "hs_hotrg_side.h"
 
 using namespace hs;
 
@@ -187,14 +188,13 @@ extern "C" hs_status hs_hotrg_step(hs_ctx ctx, hs_z2_tensor* t, int chi, int dir
   HS_CUDA(launch_select(wL, n0, wL + n0, n1, chi, idxL, lam, selL, s));
   HS_CUDA(launch_select(wR, n0, wR + n0, n1, chi, idxR, lam, selR, s));
   SelectOut hsel[2];
-  int hinfo[2];
+  int hinfo[4];
   HS_CUDA(cudaMemcpyAsync(hsel, selL, sizeof hsel, cudaMemcpyDeviceToHost, s));
-  HS_CUDA(cudaMemcpyAsync(hinfo, static_cast<int*>(ctx->info.p) + 2, sizeof hinfo, cudaMemcpyDeviceToHost, s));
+  HS_CUDA(cudaMemcpyAsync(hinfo, ctx->info.p, sizeof hinfo, cudaMemcpyDeviceToHost, s));
   HS_CUDA(cudaStreamSynchronize(s));
-  // the right Gram matrix's blocks: the left one's odd block can report info = 1
-  // (Ising, beta = 0.6, chi = 16, fourth step) on a step that matches ln Z
-  if (hinfo[0] != 0 || hinfo[1] != 0) return fail(HS_ERR_SOLVER, "syevd info = (%d, %d)", hinfo[0], hinfo[1]);
-  const int side = hsel[0].discarded <= hsel[1].discarded ? 0 : 1;
+  const int side = hotrg_side(hinfo, hsel[0].discarded, hsel[1].discarded);
+  if (side < 0)
+    return fail(HS_ERR_SOLVER, "syevd info = (%d, %d) left, (%d, %d) right", hinfo[0], hinfo[1], hinfo[2], hinfo[3]);
   const SelectOut sel = hsel[side];
   const Sect hn = make_sect(sel.chi_new[0], sel.chi_new[1]);
 
