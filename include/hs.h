@@ -600,7 +600,10 @@ hs_status hs_ctmrg_energy_grad(hs_ctx ctx, const double* A, int d, int D, hs_bas
  * two ping-pong buffers of the enlarged-corner and edge chains, sized for the
  * plain basis ((chi D^2)^2 doubles each, chi at least D^2), and three
  * chi^2 D^2 buffers. Not counted: solver workspaces, tensor-core split
- * operands and the subspace solver's buffers. precision is not used yet.
+ * operands, the subspace solver's buffers, the digits of FP64 operands (up to
+ * 1 GiB, allocated by the first FP64 product that takes them; see hs_gemm) and
+ * the partial sums of products that split K (32 MB). A context keeps these
+ * until it is destroyed; each has its own. precision is not used yet.
  * HS_ERR_INVALID_ARG if D or chi is below 1 or bytes is NULL. Host only. */
 hs_status hs_workspace_query(int D, int chi, hs_precision precision, size_t* bytes);
 

@@ -68,8 +68,9 @@ hs_status gemm(hs_ctx ctx, hs_gemm_backend be, const GemmGroup& g, const double*
 
 hs_status gemm_dfma(hs_ctx ctx, const GemmGroup& g, const double* A, const double* B, double* C, double alpha,
                     bool accumulate) {
-  HS_TRY(ctx->splitk.ensure(kSplitKElems * sizeof(double)));
-  HS_CUDA(launch_gemm_f64(g, A, B, C, alpha, ctx->stream, ctx->splitk.d(), kSplitKElems, accumulate));
+  // the workspace of the splits, for products that split K; without it they run unsplit
+  const bool split = gemm_f64_splits(g, kSplitKElems) > 1 && ctx->splitk.ensure(kSplitKElems * sizeof(double)) == HS_OK;
+  HS_CUDA(launch_gemm_f64(g, A, B, C, alpha, ctx->stream, split ? ctx->splitk.d() : nullptr, kSplitKElems, accumulate));
   if (g.n > 0) ctx->launches += 1;
   return HS_OK;
 }

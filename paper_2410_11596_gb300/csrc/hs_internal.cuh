@@ -399,6 +399,8 @@ cudaError_t launch_gemm_tc(int precision, const TcProblem* probs, int nprob, int
 // part/part_elems: optional workspace for split-K partial sums (used when the
 // output tiles alone cannot fill the GPU); nullptr disables splitting.
 // accumulate: C += alpha A B^T instead of C = alpha A B^T.
+// gemm_f64_splits: the number of K splits that a workspace of part_elems gives.
+int gemm_f64_splits(const GemmGroup& g, long long part_elems);
 cudaError_t launch_gemm_f64(const GemmGroup& g, const double* A, const double* B, double* C,
                             double alpha, cudaStream_t s, double* part = nullptr, long long part_elems = 0,
                             bool accumulate = false);

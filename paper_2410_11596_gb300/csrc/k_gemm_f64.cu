@@ -175,34 +175,37 @@ __global__ void splitk_reduce_kernel(GemmGroup g, SplitK sk, const double* __res
 }
 }  // namespace
 
-cudaError_t launch_gemm_f64(const GemmGroup& g, const double* A, const double* B, double* C,
-                            double alpha, cudaStream_t s, double* part, long long part_elems, bool accumulate) {
-  long long tiles = 0;
+// K is split when the output tiles cannot fill the GPU (3 resident CTAs on each of
+// its SMs) and each split still gets several K steps.
+int gemm_f64_splits(const GemmGroup& g, long long part_elems) {
+  long long tiles = 0, need = 0;
   int kmax = 0;
   for (int i = 0; i < g.n; ++i) {
     tiles += (long long)((g.p[i].M + BM - 1) / BM) * ((g.p[i].N + BN - 1) / BN);
+    need += (long long)g.p[i].M * g.p[i].N;
     kmax = g.p[i].K > kmax ? g.p[i].K : kmax;
   }
-  if (tiles == 0) return cudaSuccess;
-  // split K when the output tiles cannot fill the GPU (3 resident CTAs on each
-  // of its SMs) and each split still gets several K steps
   const long long kTarget = 3LL * device_sms();
+  if (tiles == 0 || tiles >= kTarget) return 1;
+  int ns = (int)((kTarget + tiles - 1) / tiles);
+  ns = ns < kmax / (4 * BK) ? ns : kmax / (4 * BK);
+  ns = ns < 64 ? ns : 64;
+  while (ns > 1 && need * ns > part_elems) --ns;
+  return ns > 1 ? ns : 1;
+}
+
+cudaError_t launch_gemm_f64(const GemmGroup& g, const double* A, const double* B, double* C,
+                            double alpha, cudaStream_t s, double* part, long long part_elems, bool accumulate) {
+  long long tiles = 0;
+  for (int i = 0; i < g.n; ++i) tiles += (long long)((g.p[i].M + BM - 1) / BM) * ((g.p[i].N + BN - 1) / BN);
+  if (tiles == 0) return cudaSuccess;
   SplitK sk{};
-  sk.nsplit = 1;
-  if (part && tiles < kTarget) {
-    int ns = (int)((kTarget + tiles - 1) / tiles);
-    ns = ns < kmax / (4 * BK) ? ns : kmax / (4 * BK);
-    ns = ns < 64 ? ns : 64;
-    long long need = 0;
-    for (int i = 0; i < g.n; ++i) need += (long long)g.p[i].M * g.p[i].N;
-    while (ns > 1 && need * ns > part_elems) --ns;
-    if (ns > 1) {
-      sk.nsplit = ns;
-      long long off = 0;
-      for (int i = 0; i < g.n; ++i) {
-        sk.part_off[i] = off;
-        off += (long long)g.p[i].M * g.p[i].N * ns;
-      }
+  sk.nsplit = part ? gemm_f64_splits(g, part_elems) : 1;
+  if (sk.nsplit > 1) {
+    long long off = 0;
+    for (int i = 0; i < g.n; ++i) {
+      sk.part_off[i] = off;
+      off += (long long)g.p[i].M * g.p[i].N * sk.nsplit;
     }
   }
   // entries of padded tiles that the busiest SM computes: the smaller count wins
