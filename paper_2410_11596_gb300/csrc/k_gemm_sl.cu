@@ -186,8 +186,9 @@ __device__ __forceinline__ void step_mmas(uint32_t leader, uint32_t tmem, uint32
 constexpr int kTileRows = BM * (BN / PART);
 static_assert(BN / PART == kEpiWarps / 4, "a warp per quarter of the rows and part of the columns");
 struct SlList {
-  int count, pad[3];
-  long long at[1];  // of kTileRows a tile
+  int count, pad;
+  unsigned long long work;  // FMAs of the entries that mag_kernel listed
+  long long at[1];          // of kTileRows a tile
 };
 
 // Appends the rows of this warp with `on`.
@@ -219,9 +220,10 @@ __device__ __forceinline__ SlTile tile_at(const SlGroup& g, int t) {
 
 template <bool ACC>
 __global__ void __launch_bounds__(NT, 1) gemm_sl_kernel(const __grid_constant__ SlGroup g, int total_tiles,
-                                                        uint32_t* __restrict__ masks,
+                                                        unsigned long long limit, uint32_t* __restrict__ masks,
                                                         SlList* __restrict__ list, int* __restrict__ err) {
   hs_pdl_enter();
+  if (list->work > limit) return;  // fma_kernel computes the whole product
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   double* stage_c = reinterpret_cast<double*>(smem + STAGES * STAGE_BYTES);
@@ -556,12 +558,80 @@ __device__ __forceinline__ void fma_row(const SlUnit& U, int row, int col0, uint
   }
 }
 
-// A listed row at a time: one warp's where the contraction is short, else one CTA's.
+// A 64 x 64 tile of a product, every entry a chain of FMAs over k, as gemm_f64_nt_kernel
+// computes it.
+constexpr int FT = 64, FK = 16;
+__device__ __forceinline__ void fma_tile(const SlUnit& U, int m0, int n0, bool accumulate, double (*As)[FT + 2],
+                                         double (*Bs)[FT + 2]) {
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  double acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  for (int k0 = 0; k0 < U.K; k0 += FK) {
+    const int k = k0 + tx, s = k >= U.a.kseg, ks = s ? k - U.a.kseg : k;
+    const bool in = k < U.K, flip = in && U.a.neg[s] != U.b.neg[s];
+    const double* pa = (s ? U.a.p[1] : U.a.p[0]) + ks;
+    const double* pb = (s ? U.b.p[1] : U.b.p[0]) + ks;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = ty + 16 * i;
+      const double x = in && m0 + r < U.M ? pa[(long long)(m0 + r) * U.a.ld] : 0.0;
+      As[tx][r] = flip ? -x : x;
+      Bs[tx][r] = in && n0 + r < U.N ? pb[(long long)(n0 + r) * U.b.ld] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < FK; ++kk) {
+      double a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        a[i] = As[kk][ty + 16 * i];
+        b[i] = Bs[kk][tx + 16 * i];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
+      if (m < U.M && n < U.N) {
+        double* o = U.c + (long long)m * U.ldc + n;
+        *o = accumulate ? *o + acc[i][j] : acc[i][j];
+      }
+    }
+}
+
+// A listed row at a time: one warp's where the contraction is short, else one CTA's. Where
+// the listed entries are more than a third of the work (limit), which the rows' FMAs take
+// as long for as the whole product takes on shared tiles, the whole product is computed
+// that way and gemm_sl_kernel is left out: 10368 x 666 x 666 with every entry listed
+// 8.4 ms (23.2 row by row, 19.1 as serial dot products in the epilogue; the FP64 kernel alone
+// 8.0), one column of NaN 0.49 ms (1.66).
 constexpr int kWarpK = 512;
-__global__ void __launch_bounds__(256) fma_kernel(const __grid_constant__ SlGroup g, bool accumulate,
-                                                  const uint32_t* __restrict__ masks, const SlList* __restrict__ list) {
+__global__ void __launch_bounds__(256, 3) fma_kernel(const __grid_constant__ SlGroup g, bool accumulate,
+                                                     unsigned long long limit, const uint32_t* __restrict__ masks,
+                                                     const SlList* __restrict__ list) {
   hs_pdl_enter();
   __shared__ double red[8][4];
+  __shared__ double As[FK][FT + 2], Bs[FK][FT + 2];
+  if (list->work > limit) {
+    int t = blockIdx.x;
+    for (int u = 0; u < g.n; ++u) {
+      const SlUnit& U = g.u[u];
+      const int tn = (U.N + FT - 1) / FT, tiles = (U.M + FT - 1) / FT * tn;
+      for (; t < tiles; t += gridDim.x) fma_tile(U, t / tn * FT, t % tn * FT, accumulate, As, Bs);
+      t -= tiles;
+    }
+    return;
+  }
   const int n = list->count;
   bool longer = false, shorter = false;
   for (int u = 0; u < g.n; ++u) (g.u[u].K > kWarpK ? longer : shorter) = true;
@@ -747,13 +817,17 @@ __global__ void __launch_bounds__(MNT, 2) mag_kernel(const __grid_constant__ SlG
         const float low = U.g_low * sqrtf(fminf(ra.count, nb) * inv_k);
         if (S > 0.f && S < U.g_round * (fminf(ra.sum, nb) + fminf(sb, ra.count)) + low) again |= 1ull << j;
       }
+      unsigned entries = 0u;
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         const uint32_t m = row < U.M ? (uint32_t)(again >> (p * PART)) & part_columns(U.N - col0 - p * PART) : 0u;
         const long long at = ((long long)t * BM + q * 32 + lane) * (BN / PART) + 2 * half + p;
         masks[at] = m;
         list_rows(list, m != 0u, at);
+        entries += __popc(m);
       }
+      entries = __reduce_add_sync(0xffffffffu, entries);
+      if (lane == 0 && entries != 0u) atomicAdd(&list->work, (unsigned long long)entries * U.K);
     }
   }
   fence_before();
@@ -970,7 +1044,10 @@ template <int NR>
 __global__ void __launch_bounds__(256) slice_split_kernel(const __grid_constant__ SplitOps ops, int T) {
   hs_pdl_enter();
   const SplitOp& P = ops.op[blockIdx.y];
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) ops.list->count = 0;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    ops.list->count = 0;
+    ops.list->work = 0ull;
+  }
   const int Kp = P.steps * KC;
   // 16-byte loads: even strides and lengths, sources aligned and changing between pieces
   const bool vec = P.K % 2 == 0 && P.m.ld % 2 == 0 && (reinterpret_cast<uintptr_t>(P.m.p[0]) & 15) == 0 &&
@@ -1238,8 +1315,17 @@ cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* pro
   if (e != cudaSuccess) return e;
   uint32_t* const masks = reinterpret_cast<uint32_t*>(list->at + rows);
   hs_launch(mag_kernel, (unsigned)(tiles < 2 * sms ? tiles : 2 * sms), MNT, MSMEM, s, g, tiles, masks, list, err);
-  hs_launch(gemm, (unsigned)(tiles < sms ? tiles : sms), NT, SMEM, s, g, tiles, masks, list, err);
-  hs_launch(fma_kernel, (unsigned)(4 * sms), 256, 0, s, g, accumulate, (const uint32_t*)masks, (const SlList*)list);
+  // a third of the work, where the product has tiles enough for fma_kernel's CTAs
+  unsigned long long fmas = 0;
+  long long tiles64 = 0;
+  for (int i = 0; i < g.n; ++i) {
+    fmas += (unsigned long long)g.u[i].M * g.u[i].N * g.u[i].K;
+    tiles64 += (long long)((g.u[i].M + FT - 1) / FT) * ((g.u[i].N + FT - 1) / FT);
+  }
+  const unsigned long long limit = tiles64 >= 2 * sms && tiles64 < INT_MAX / 2 ? fmas / 3 : ~0ull;
+  hs_launch(gemm, (unsigned)(tiles < sms ? tiles : sms), NT, SMEM, s, g, tiles, limit, masks, list, err);
+  hs_launch(fma_kernel, (unsigned)(4 * sms), 256, 0, s, g, accumulate, limit, (const uint32_t*)masks,
+            (const SlList*)list);
   return cudaGetLastError();
 }
 
