@@ -527,7 +527,7 @@ hs_status hs_profile_read(hs_ctx ctx, double* phase_ms, double* phase_flops, int
  * kernel, or, where the product is large enough to pay for it, sums of exact
  * digit products on the tensor cores; either way the error of an entry stays
  * below the bound of a chain of FP64 FMAs, K 2^-53 sum_k |A_mk| |B_nk| (entries
- * that the digits cannot hold to 4 sqrt(K) 2^-53 of that sum are summed by FMAs;
+ * that the digits cannot hold to 2 sqrt(K) 2^-53 of that sum are summed by FMAs;
  * no digits on a stream under capture; the operands' digits are kept in the
  * context workspace, at most 1 GiB); the TF32/BF16 modes split A and B into hi/lo parts (padded copies in
  * the context workspace) and run the tcgen05 tensor-core kernel with FP32
