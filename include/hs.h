@@ -607,6 +607,22 @@ hs_status hs_ctmrg_energy_grad(hs_ctx ctx, const double* A, int d, int D, hs_bas
  * HS_ERR_INVALID_ARG if D or chi is below 1 or bytes is NULL. Host only. */
 hs_status hs_workspace_query(int D, int chi, hs_precision precision, size_t* bytes);
 
+/* Diagnostic: one FP64 product of the library's chains, C = A B^T (M x N, contraction
+ * K, contiguous rows) or C += A B^T (accumulate), or with all of Ai, Bi and Ci
+ * the complex product of planar parts, C = A B^T or A conj(B)^T (conj_b), with
+ * the digits' workspace limited to slice_bytes (0: as if none could be had), so
+ * that a test reaches the panels of large products at small sizes. *panels (host):
+ * the pairs of row panels that the product took, 1 whole, 0 not by digits.
+ * Asynchronous. */
+hs_status hs_selftest_gemm_f64(hs_ctx ctx, int M, int N, int K, const double* Ar, const double* Ai, const double* Br,
+                               const double* Bi, double* Cr, double* Ci, int conj_b, int accumulate, size_t slice_bytes,
+                               int* panels);
+
+/* Diagnostic: the number of eigensolvers (4, the default, or 2) that
+ * hs_hotrg_step runs at once on this context; 2 is what a step falls back to
+ * where the other two cannot be had. Host only. */
+hs_status hs_selftest_hotrg_solvers(hs_ctx ctx, int at_once);
+
 /* Diagnostic: runs the tensor-core GEMM's bounded mbarrier wait (the wait
  * every pipeline stage of that kernel uses, which gives up after a fixed
  * number of try_wait rounds, raises the kernel's abort flag and records an

@@ -123,6 +123,9 @@ _PROTOS = {
     "hs_ctmrg4_move": (c_int, [c_void_p, POINTER(Z2Tensor), POINTER(Env4), c_int, c_int, POINTER(Move4Info),
                                POINTER(c_double)]),
     "hs_env4_to_dense": (c_int, [c_void_p, POINTER(Env4), POINTER(c_void_p), POINTER(c_void_p)]),
+    "hs_selftest_gemm_f64": (c_int, [c_void_p, c_int, c_int, c_int] + [c_void_p] * 6 + [c_int, c_int, c_size_t,
+                                     POINTER(c_int)]),
+    "hs_selftest_hotrg_solvers": (c_int, [c_void_p, c_int]),
     "hs_selftest_bounded_wait": (c_int, [c_void_p, ctypes.c_longlong, POINTER(c_int)]),
     "hs_hotrg_tensor_bytes": (c_size_t, [c_int, c_int]),
     "hs_hotrg_init": (c_int, [c_void_p, POINTER(Z2Tensor), POINTER(Z2Tensor), POINTER(c_double)]),
@@ -271,6 +274,22 @@ def hs_ctmrg4_move(ctx: int, a: Z2Tensor, env: Env4, chi: int, direction: int) -
 def hs_env4_to_dense(ctx: int, env: Env4, C_dense, T_dense) -> None:
     check(load().hs_env4_to_dense(ctx, ctypes.byref(env), (c_void_p * 4)(*[ptr(x) for x in C_dense]),
                                   (c_void_p * 4)(*[ptr(x) for x in T_dense])))
+
+
+def hs_selftest_gemm_f64(ctx: int, A, B, C, slice_bytes: int, conj_b: bool = False, accumulate: bool = False) -> int:
+    """C (+)= A B^T; A, B, C each a tensor or a (real, imaginary) pair. Returns the panel pairs taken."""
+    Ar, Ai = A if isinstance(A, tuple) else (A, None)
+    Br, Bi = B if isinstance(B, tuple) else (B, None)
+    Cr, Ci = C if isinstance(C, tuple) else (C, None)
+    n = c_int()
+    opt = lambda t: ptr(t) if t is not None else None
+    check(load().hs_selftest_gemm_f64(ctx, Ar.shape[0], Br.shape[0], Ar.shape[1], ptr(Ar), opt(Ai), ptr(Br), opt(Bi),
+                                      ptr(Cr), opt(Ci), conj_b, accumulate, slice_bytes, ctypes.byref(n)))
+    return n.value
+
+
+def hs_selftest_hotrg_solvers(ctx: int, at_once: int) -> None:
+    check(load().hs_selftest_hotrg_solvers(ctx, at_once))
 
 
 def hs_selftest_bounded_wait(ctx: int, limit: int) -> list[int]:

@@ -76,10 +76,6 @@ hs_status gemm_dfma(hs_ctx ctx, const GemmGroup& g, const double* A, const doubl
 }
 
 namespace {
-// The digit slices' workspace per context, at most. Larger products run in
-// panels of rows whose slices fill half of it (the other operand's in the rest).
-constexpr size_t kSliceBytes = size_t(1) << 30;
-
 // A stream under capture gets the FP64 kernel: it needs no workspace that a
 // later call could outgrow while the graph still points to it.
 bool capturing(cudaStream_t s) {
@@ -110,11 +106,37 @@ int operand(SlMat* mats, int* n, const SlMat& m) {
   return (*n)++;
 }
 
+// Rows of a panel of each operand in `room` bytes: the smaller operand in one panel if
+// that takes no more than 3/8 of the room, the other in what is left of 3/4, the list of a
+// panel pair's entries in the last quarter. False if not even a block of rows fits.
+bool panel_rows(const SlMat& a, const SlMat& b, size_t room, int* ra, int* rb) {
+  auto rows = [](const SlMat& x, size_t bytes) {
+    const int block = slices_block(x.is_b);
+    const long long r = (long long)(bytes / slices_bytes(block, x.kseg * x.nseg, x.is_b)) * block;
+    return (int)(r < x.rows ? r : x.rows);
+  };
+  auto size = [](const SlMat& x, int r) { return slices_bytes(r, x.kseg * x.nseg, x.is_b); };
+  *ra = rows(a, room / 8 * 3);
+  *rb = rows(b, room / 8 * 3);
+  if (*ra < 1 || *rb < 1) return false;
+  if (*rb == b.rows)
+    *ra = rows(a, room / 4 * 3 - size(b, *rb));
+  else if (*ra == a.rows)
+    *rb = rows(b, room / 4 * 3 - size(a, *ra));
+  // whole waves of tiles
+  const int ba = slices_block(false), tn = (*rb + slices_block(true) - 1) / slices_block(true);
+  const int sms = device_sms(), waves = (*ra / ba) * tn / sms;
+  if (*ra < a.rows && tn <= sms && waves > 0) *ra = waves * sms / tn * ba;
+  while (*ra > ba && slices_list_bytes(*ra, *rb) > room / 4) *ra = std::max(ba, *ra / 2 / ba * ba);
+  return slices_list_bytes(*ra, *rb) <= room / 4;
+}
+
 // The products on the tensor cores by digit slices when that is the faster
 // way; *done = false leaves them to the FP64 kernel.
 hs_status gemm_sliced(hs_ctx ctx, const SlMat* mats, int nm, const SlProblem* probs, int np,
                       bool accumulate, bool* done) {
   *done = false;
+  ctx->sl_panels = 0;
   if (np < 1 || ctx->no_slices || !slices_pay(probs, mats, np) || capturing(ctx->stream)) return HS_OK;
   SlMat m[2 * kMaxProblems];
   size_t scales = 0, all = 0;
@@ -126,45 +148,40 @@ hs_status gemm_sliced(hs_ctx ctx, const SlMat* mats, int nm, const SlProblem* pr
   }
   for (int i = 0; i < np; ++i) all += slices_list_bytes(m[probs[i].a].rows, m[probs[i].b].rows);
   all += scales;
-  if (ctx->sl_ws.ensure(all < kSliceBytes ? all : kSliceBytes) != HS_OK) return HS_OK;  // no memory left
+  const size_t want = std::min(all, ctx->sl_cap);
+  if (want <= scales) return HS_OK;
+  const size_t room = want - scales;
+  int ra[kMaxProblems], rb[kMaxProblems];
+  if (all > want)
+    for (int i = 0; i < np; ++i)
+      if (!panel_rows(m[probs[i].a], m[probs[i].b], room, &ra[i], &rb[i])) return HS_OK;
+  if (ctx->sl_ws.ensure(want) != HS_OK) return HS_OK;  // no memory left
   int* err = static_cast<int*>(ctx->tc_err.p);
   char* const ws = static_cast<char*>(ctx->sl_ws.p) + scales;
-  const size_t room = ctx->sl_ws.bytes - scales;
   HS_CUDA(launch_slice_scales(m, nm, probs, np, ctx->sl_ws.p, ctx->stream));
   ctx->launches += 1;
   *done = true;
-  if (all <= ctx->sl_ws.bytes) {
+  if (all <= want) {
     HS_CUDA(launch_gemm_slices(m, nm, probs, np, accumulate, ws, room, err, ctx->stream));
     ctx->launches += 4;
+    ctx->sl_panels = 1;
     return HS_OK;
   }
   for (int i = 0; i < np; ++i) {
     const SlMat &a = m[probs[i].a], &b = m[probs[i].b];
-    // the smaller operand in one panel if that takes no more than 3/8 of the room, the
-    // other in what is left of 3/4; the list of a panel's entries in the last quarter
-    auto rows = [](const SlMat& x, size_t bytes) {
-      const int block = slices_block(x.is_b);
-      const long long r = (long long)(bytes / slices_bytes(block, x.kseg * x.nseg, x.is_b)) * block;
-      return (int)(r < x.rows ? r : x.rows);
-    };
-    auto size = [](const SlMat& x, int r) { return slices_bytes(r, x.kseg * x.nseg, x.is_b); };
-    int ra = rows(a, room / 8 * 3), rb = rows(b, room / 8 * 3);
-    if (rb == b.rows)
-      ra = rows(a, room / 4 * 3 - size(b, rb));
-    else if (ra == a.rows)
-      rb = rows(b, room / 4 * 3 - size(a, ra));
-    // whole waves of tiles
-    const int ba = slices_block(false), tn = (rb + slices_block(true) - 1) / slices_block(true);
-    const int sms = device_sms(), waves = (ra / ba) * tn / sms;
-    if (ra < a.rows && tn <= sms && waves > 0) ra = waves * sms / tn * ba;
-    while (ra > ba && slices_list_bytes(ra, rb) > room / 4) ra = std::max(ba, ra / 2 / ba * ba);
-    if (ra < 1 || rb < 1) return fail(HS_ERR_SHAPE, "contraction of %d too long for the slices", a.kseg * a.nseg);
-    for (int n0 = 0; n0 < b.rows; n0 += rb)
-      for (int m0 = 0; m0 < a.rows; m0 += ra) {
-        const SlMat part[2] = {row_panel(a, m0, std::min(ra, a.rows - m0)), row_panel(b, n0, std::min(rb, b.rows - n0))};
-        const SlProblem pr = {0, 1, probs[i].c + (long long)m0 * probs[i].ldc + n0, probs[i].ldc};
+    // the digits of a panel that the next pair has too stay where they are, first in the
+    // workspace: all of A, or the panel of B that the panels of A pass by
+    const bool keep_a = ra[i] >= a.rows;
+    for (int n0 = 0; n0 < b.rows; n0 += rb[i])
+      for (int m0 = 0; m0 < a.rows; m0 += ra[i]) {
+        SlMat part[2] = {row_panel(a, m0, std::min(ra[i], a.rows - m0)), row_panel(b, n0, std::min(rb[i], b.rows - n0))};
+        part[0].kept = keep_a && n0 > 0;
+        part[1].kept = !keep_a && m0 > 0;
+        if (!keep_a) std::swap(part[0], part[1]);
+        const SlProblem pr = {keep_a ? 0 : 1, keep_a ? 1 : 0, probs[i].c + (long long)m0 * probs[i].ldc + n0, probs[i].ldc};
         HS_CUDA(launch_gemm_slices(part, 2, &pr, 1, accumulate, ws, room, err, ctx->stream));
         ctx->launches += 4;
+        ctx->sl_panels += 1;
       }
   }
   return HS_OK;
@@ -386,6 +403,7 @@ hs_status eig_pair(hs_ctx ctx, bool f32, void* A0, int n0, void* w0, void* A1, i
 }
 static hs_status quad_lanes(hs_ctx ctx, int nmax) {
   int i = 2;
+  if (!ctx->use_lanes) return HS_ERR_UNSUPPORTED;
   for (hs_ctx_s::Lane& l : ctx->lane) {
     if (!l.stream) HS_CUDA(cudaStreamCreateWithFlags(&l.stream, cudaStreamNonBlocking));
     if (!l.join) HS_CUDA(cudaEventCreateWithFlags(&l.join, cudaEventDisableTiming));
@@ -1865,6 +1883,32 @@ hs_status hs_env_bytes(int D, int chi_max, size_t* C_bytes, size_t* T_bytes) {
   const size_t chi = (size_t)(chi_max > D * D ? chi_max : D * D);
   *C_bytes = chi * chi * sizeof(double);
   *T_bytes = chi * (size_t)D * D * chi * sizeof(double);
+  return HS_OK;
+}
+
+hs_status hs_selftest_gemm_f64(hs_ctx ctx, int M, int N, int K, const double* Ar, const double* Ai, const double* Br,
+                               const double* Bi, double* Cr, double* Ci, int conj_b, int accumulate, size_t slice_bytes,
+                               int* panels) {
+  HS_TRY(check_ctx(ctx));
+  const bool cx = Ai || Bi || Ci;
+  if (M < 1 || N < 1 || K < 1 || !Ar || !Br || !Cr || (cx && (!Ai || !Bi || !Ci || accumulate)) || !panels)
+    return fail(HS_ERR_INVALID_ARG, "bad arguments");
+  GemmGroup g{};
+  g.n = 1;
+  g.p[0] = GemmProblem{M, N, K, K, K, N, 0, 0, 0};
+  const size_t cap = ctx->sl_cap;
+  ctx->sl_cap = std::min(cap, slice_bytes);
+  const hs_status st = cx ? zgemm_f64(ctx, g, Ar, Ai, Br, Bi, Cr, Ci, conj_b != 0)
+                          : gemm_f64(ctx, g, Ar, Br, Cr, accumulate != 0);
+  ctx->sl_cap = cap;
+  *panels = ctx->sl_panels;
+  return st;
+}
+
+hs_status hs_selftest_hotrg_solvers(hs_ctx ctx, int at_once) {
+  HS_TRY(check_ctx(ctx));
+  if (at_once != 2 && at_once != 4) return fail(HS_ERR_INVALID_ARG, "two or four solvers");
+  ctx->use_lanes = at_once == 4;
   return HS_OK;
 }
 

@@ -168,6 +168,7 @@ struct hs_ctx_s {
     hs::DBuf dev;
     std::vector<char> host;
   } lane[2];
+  bool use_lanes = true;  // (off: one pair of solves after the other, as where they cannot be had)
   // HOTRG workspace
   hs::DBuf hb[16];
   // complex (graded) CTMRG: private copy of a~ followed by its conjugate, and scratch
@@ -189,6 +190,10 @@ struct hs_ctx_s {
   // split-K partial sums of the FP64 GEMM, digit slices of its operands
   hs::DBuf splitk, sl_ws;
   bool no_slices = false;  // this call's FP64 products all take the FP64 kernel (NoSlices)
+  // the digit slices' workspace, at most. Larger products run in panels of rows
+  // whose slices fit it (a self-test lowers it to reach them).
+  size_t sl_cap = size_t(1) << 30;
+  int sl_panels = 0;  // panel pairs of the last FP64 product (1: whole, 0: not by slices)
   // subspace eigensolver: warm start (previous kept rows, per block) and
   // per-block iteration buffers
   const void* ws_env = nullptr;

@@ -416,6 +416,7 @@ struct SlMat {
   long long ld;
   bool is_b;  // an N-side operand (its digit planes are laid out in other row blocks)
   const short* scale = nullptr;  // scales of the columns (launch_slice_scales)
+  bool kept = false;  // its slices are in the workspace already, from the call before
 };
 // C[rows of mats[a], rows of mats[b]] = A B^T (+ C).
 struct SlProblem {

@@ -1220,11 +1220,12 @@ cudaError_t launch_slice_scales(SlMat* mats, int nmat, const SlProblem* probs, i
 cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob, bool accumulate,
                                void* ws, size_t ws_bytes, int* err, cudaStream_t s) {
   if (nmat > kMaxSplit || nprob > kMaxProblems || nprob < 1) return cudaErrorInvalidValue;
-  SplitOps ops{};
+  SplitOp all[kMaxSplit] = {};
+  SplitOps ops{};  // of the operands to be split
   size_t off = 0;
-  int rmax = 0, kmax = 0;
+  int rmax = 0, kmax = 0, nsplit = 0;
   for (int i = 0; i < nmat; ++i) {
-    SplitOp& o = ops.op[i];
+    SplitOp& o = all[i];
     if (!mats[i].scale) return cudaErrorInvalidValue;
     o.m = mats[i];
     o.scale = mats[i].scale;
@@ -1239,15 +1240,18 @@ cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* pro
     off += up256((size_t)o.m.rows * sizeof(int));
     o.row = reinterpret_cast<SlRow*>(static_cast<char*>(ws) + off);
     off += up256((size_t)o.m.rows * sizeof(SlRow));
+    if (mats[i].kept) continue;
+    ops.op[nsplit++] = o;
     rmax = o.m.rows > rmax ? o.m.rows : rmax;
     kmax = o.K > kmax ? o.K : kmax;
   }
+  if (nsplit < 1) return cudaErrorInvalidValue;
   SlList* const list = reinterpret_cast<SlList*>(static_cast<char*>(ws) + off);
   ops.list = list;
   SlGroup g{};
   int tiles = 0;
   for (int i = 0; i < nprob; ++i) {
-    const SplitOp &a = ops.op[probs[i].a], &b = ops.op[probs[i].b];
+    const SplitOp &a = all[probs[i].a], &b = all[probs[i].b];
     if (a.K != b.K || a.m.kseg != b.m.kseg || a.K < 1 || a.m.rows < 1 || b.m.rows < 1 || a.block != BM ||
         b.block != BN)
       return cudaErrorInvalidValue;
@@ -1299,7 +1303,7 @@ cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* pro
   const int nr = (pieces + T - 1) / T, per = 256 / T;
   int gx = (rmax + per - 1) / per;
   if (gx > sms * 32) gx = sms * 32;
-  const dim3 grid((unsigned)gx, (unsigned)nmat);
+  const dim3 grid((unsigned)gx, (unsigned)nsplit);
   if (nr == 1)
     hs_launch(slice_split_kernel<1>, grid, 256, 0, s, ops, T);
   else if (nr == 2)
