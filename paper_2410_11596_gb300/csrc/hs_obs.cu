@@ -492,7 +492,13 @@ __global__ void site_sum_kernel(const double* __restrict__ pk, const double* __r
 struct ZBuf {
   double* re;
   double* im;
+  ZBuf at(long long n) const { return {re + n, im ? im + n : nullptr}; }
 };
+
+// The largest intermediates, c^2 d^2 q^2 entries, are made a few of their leading
+// index's values at a time where they would hold more than this (4 GB a part): at d = 2,
+// D = 6, c = 144 they hold 0.9 GB, at d = 16, D = 7, c = 196 two of them were 378 GB.
+constexpr long long kObsElems = 1ll << 29;
 
 // One observable's evaluation: real or complex arithmetic on the context's buffers.
 struct Obs {
@@ -619,26 +625,32 @@ SiteLegs site_legs(bool cx, bool left) {
 }
 
 // A site's half network out[(x0, S, S') | x4], S = (s, m): Xp[(x0, e, k0b, k1b) | (k0k, k1k)]
-// with the ket tensor, the bra tensor and the edge T[e, k2, x4].
+// with the ket tensor, the bra tensor and the edge T[e, k2, x4]. Every step keeps x0
+// outermost, so that it runs on ranges of x0 (kObsElems).
 hs_status site_half(const Obs& o, ZBuf Xp, const SiteLegs& g, ZBuf out) {
   const long long c = o.c, D = o.D, q = o.q, S = o.d * D;
   ZBuf A, AP, T, TB, Y1, Y1p, Y2, Xf;
-  const long long n1 = c * c * q * S * D, n2 = c * c * S * D * S * D;
+  const long long per = c * S * D * (q > S * D ? q : S * D);  // entries a value of x0
+  const long long cb = kObsElems / per > c ? c : kObsElems / per > 0 ? kObsElems / per : 1;
   HS_TRY(o.buf(bA, S * D * q, &A));
   HS_TRY(o.buf(bT, c * q * c, &T));
   HS_TRY(o.buf(bScratch + 1, S * D * q, &AP));
   HS_TRY(o.buf(bScratch + 2, c * q * c, &TB));
-  HS_TRY(o.buf(bScratch + 3, n2 > n1 ? n2 : n1, &Y1));
-  HS_TRY(o.buf(bScratch + 4, n2 > n1 ? n2 : n1, &Y1p));
+  HS_TRY(o.buf(bScratch + 3, cb * per, &Y1));
+  HS_TRY(o.buf(bScratch + 4, cb * per, &Y1p));
   Y2 = Y1;
   Xf = Y1p;
   HS_TRY(o.perm(dense({o.d, D, D, D}, {D}), dense({o.d, D, D}, {D, D}), {0, g.m, g.k2, g.k0, g.k1}, A, AP));
   HS_TRY(o.perm(dense({c, D, D}, {c}), dense({c}, {c, D, D}), {3, 0, 2, 1}, T, TB));              // [x4 | (e, k2k, k2b)]
-  HS_TRY(o.mul(c * c * q, S * D, q, Xp, AP, Y1));                                                  // [(x0, e, k0b, k1b) | (S, k2k)]
-  HS_TRY(o.perm(dense({c * c, q}, {S * D}), dense({c * c, S * D}, {q}), {0, 2, 1}, Y1, Y1p));      // [(x0, e, S, k2k) | (k0b, k1b)]
-  HS_TRY(o.mul(c * c * S * D, S * D, q, Y1p, AP, Y2, true));                                       // [(x0, e, S, k2k) | (S', k2b)]
-  HS_TRY(o.perm(dense({c, c, S, D}, {S, D}), dense({c, S, S}, {c, D, D}), {0, 2, 4, 1, 3, 5}, Y2, Xf));
-  return o.mul(c * S * S, c, c * q, Xf, TB, out);
+  for (long long x0 = 0; x0 < c; x0 += cb) {
+    const long long b = c - x0 < cb ? c - x0 : cb;
+    HS_TRY(o.mul(b * c * q, S * D, q, Xp.at(x0 * c * q * q), AP, Y1));                               // [(x0, e, k0b, k1b) | (S, k2k)]
+    HS_TRY(o.perm(dense({b * c, q}, {S * D}), dense({b * c, S * D}, {q}), {0, 2, 1}, Y1, Y1p));      // [(x0, e, S, k2k) | (k0b, k1b)]
+    HS_TRY(o.mul(b * c * S * D, S * D, q, Y1p, AP, Y2, true));                                       // [(x0, e, S, k2k) | (S', k2b)]
+    HS_TRY(o.perm(dense({b, c, S, D}, {S, D}), dense({b, S, S}, {c, D, D}), {0, 2, 4, 1, 3, 5}, Y2, Xf));
+    HS_TRY(o.mul(b * S * S, c, c * q, Xf, TB, out.at(x0 * S * S * c)));
+  }
+  return HS_OK;
 }
 
 // Forward chain of the two-site network: leaves T (bT), the ring V (bV, [(e, k0) | (x0, k1)]
@@ -718,9 +730,11 @@ hs_status finish_rdm(hs_ctx ctx, const hs_env* env, int d, int D, const double* 
 hs_status rdm_vjp_after_chain(hs_ctx ctx, const hs_env* env, int d, int D, const double* A, const double* drho,
                               double* dA_out) {
   const Obs o = make_obs(ctx, env, d, D);
-  const long long c = o.c, q = o.q, S = (long long)d * D, nh = c * c * S * S, nx = c * c * q * q, nf = c * S * S * c * q,
+  const long long c = o.c, q = o.q, S = (long long)d * D, nh = c * c * S * S, nx = c * c * q * q, per = c * S * c * q,
                   nq = S * S * q * q * q;
-  ZBuf T, V, half[2], dh, dht, TT, Vt, F, Fp, Q, pp;
+  const long long sb = kObsElems / per > S ? S : kObsElems / per > 0 ? kObsElems / per : 1;  // values of S at a time
+  const long long nf = sb * per;
+  ZBuf T, V, half[2], dh, dht, dS, TT, Vt, F, Fp, Q;
   HS_TRY(o.buf(bT, c * q * c, &T));
   HS_TRY(o.buf(bV, nx, &V));
   HS_TRY(o.buf(bL, nh, &half[0]));
@@ -732,6 +746,7 @@ hs_status rdm_vjp_after_chain(hs_ctx ctx, const hs_env* env, int d, int D, const
   HS_TRY(o.buf(bScratch + 5, nh, &dh));
   HS_TRY(o.buf(bScratch + 6, nq, &Q));
   HS_TRY(o.buf(bScratch + 7, nh, &dht));
+  if (sb < S) HS_TRY(o.buf(bScratch + 8, nh, &dS));
   const int cx = o.cx ? 2 : 1;
   const long long rows = S * S * q, npart = rows * q * cx;
   HS_TRY(ctx->hb[0].ensure(2 * npart * 8));
@@ -757,9 +772,19 @@ hs_status rdm_vjp_after_chain(hs_ctx ctx, const hs_env* env, int d, int D, const
       HS_TRY(o.perm(dense({c, S * S}, {c}), dense({c, S * S}, {c}), {2, 1, 0}, dh, dht));
       din = dht;
     }
-    HS_TRY(o.mul(c * S * S, c * q, c, din, TT, F, true));  // [(x0, S, S') | (e, k2k, k2b)]
-    HS_TRY(o.perm(dense({c, S, S}, {c, D, D}), dense({S, S, D, D}, {c, c}), {1, 2, 4, 5, 0, 3}, F, Fp));
-    HS_TRY(o.mul(rows, q * q, c * c, Fp, Vt, Q, true));  // [(S, S', k2k, k2b) | (k0, k1)]
+    if (sb >= S) {
+      HS_TRY(o.mul(c * S * S, c * q, c, din, TT, F, true));  // [(x0, S, S') | (e, k2k, k2b)]
+      HS_TRY(o.perm(dense({c, S, S}, {c, D, D}), dense({S, S, D, D}, {c, c}), {1, 2, 4, 5, 0, 3}, F, Fp));
+      HS_TRY(o.mul(rows, q * q, c * c, Fp, Vt, Q, true));  // [(S, S', k2k, k2b) | (k0, k1)]
+    } else {  // the same with S outermost, on ranges of it
+      HS_TRY(o.perm(dense({c, S, S}, {c}), dense({S, c, S}, {c}), {1, 0, 2, 3}, din, dS));
+      for (long long s0 = 0; s0 < S; s0 += sb) {
+        const long long b = S - s0 < sb ? S - s0 : sb;
+        HS_TRY(o.mul(b * c * S, c * q, c, dS.at(s0 * c * S * c), TT, F, true));
+        HS_TRY(o.perm(dense({b, c, S}, {c, D, D}), dense({b, S, D, D}, {c, c}), {0, 2, 4, 5, 1, 3}, F, Fp));
+        HS_TRY(o.mul(b * S * q, q * q, c * c, Fp, Vt, Q.at(s0 * S * q * q * q), true));
+      }
+    }
     hs_launch(site_adjoint_kernel, (unsigned)rows, 64, sm, ctx->stream, (const double*)Q.re, (const double*)Q.im, A, d,
               D, g, staged, pk, pb);
     HS_CUDA(cudaGetLastError());
