@@ -162,7 +162,7 @@ hs_status gemm_sliced(hs_ctx ctx, const SlMat* mats, int nm, const SlProblem* pr
   ctx->launches += 1;
   *done = true;
   if (all <= want) {
-    HS_CUDA(launch_gemm_slices(m, nm, probs, np, accumulate, ws, room, err, ctx->stream));
+    HS_CUDA(launch_gemm_slices(m, nm, probs, np, ctx->sl_bound, accumulate, ws, room, err, ctx->stream));
     ctx->launches += 4;
     ctx->sl_panels = 1;
     return HS_OK;
@@ -179,7 +179,7 @@ hs_status gemm_sliced(hs_ctx ctx, const SlMat* mats, int nm, const SlProblem* pr
         part[1].kept = !keep_a && m0 > 0;
         if (!keep_a) std::swap(part[0], part[1]);
         const SlProblem pr = {keep_a ? 0 : 1, keep_a ? 1 : 0, probs[i].c + (long long)m0 * probs[i].ldc + n0, probs[i].ldc};
-        HS_CUDA(launch_gemm_slices(part, 2, &pr, 1, accumulate, ws, room, err, ctx->stream));
+        HS_CUDA(launch_gemm_slices(part, 2, &pr, 1, ctx->sl_bound, accumulate, ws, room, err, ctx->stream));
         ctx->launches += 4;
         ctx->sl_panels += 1;
       }
@@ -2408,6 +2408,7 @@ hs_status hs_gemm(hs_ctx ctx, hs_precision precision, int M, int N, int K, const
     g.n = 1;
     g.p[0] = GemmProblem{M, N, K, lda, ldb, ldc, 0, 0, 0};
     bool done = false;
+    const SlicesKeep bound(ctx, kBoundEntry);
     HS_TRY(gemm_try_sliced(ctx, g, A, B, C, false, &done));
     if (done) return HS_OK;
     // (split K needs the context's workspace, which a capture may not allocate)

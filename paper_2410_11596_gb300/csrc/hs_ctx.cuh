@@ -193,6 +193,7 @@ struct hs_ctx_s {
   // the digit slices' workspace, at most. Larger products run in panels of rows
   // whose slices fit it (a self-test lowers it to reach them).
   size_t sl_cap = size_t(1) << 30;
+  hs::SliceBound sl_bound = hs::kBoundChain;
   int sl_panels = 0;  // panel pairs of the last FP64 product (1: whole, 0: not by slices)
   // subspace eigensolver: warm start (previous kept rows, per block) and
   // per-block iteration buffers
@@ -262,6 +263,13 @@ struct NoSlices {
   hs_ctx c;
   NoSlices(hs_ctx ctx, bool off) : c(ctx) { c->no_slices = off; }
   ~NoSlices() { c->no_slices = false; }
+};
+// While it lives (one call), the bound that the context's sliced products keep.
+struct SlicesKeep {
+  hs_ctx c;
+  SliceBound was;
+  SlicesKeep(hs_ctx ctx, SliceBound b) : c(ctx), was(ctx->sl_bound) { c->sl_bound = b; }
+  ~SlicesKeep() { c->sl_bound = was; }
 };
 Sect q_sect(int D, hs_basis b);
 Z2Mat mat(Fused r, Fused c, int pad = 1);

@@ -431,12 +431,18 @@ size_t slices_scale_bytes(int K);
 size_t slices_list_bytes(long long M, long long N);
 int slices_block(bool is_b);  // rows per block of the planes
 bool slices_pay(const SlProblem* probs, const SlMat* mats, int n);
+// What the error of a product's entry is held to (k_gemm_sl.cu):
+enum SliceBound {
+  kBoundEntry,  // 2 sqrt(K) 2^-53 S, S = sum |a||b| of the entry: about a chain's own error
+  kBoundChain,  // K 2^-53 S: a chain's worst case
+  kBoundRows    // K 2^-55 of the largest |a| in its row times the largest |b|, after the columns' scales
+};
 // Fills the operands' scales, in ws (their slices_scale_bytes), for a following launch_gemm_slices of
 // them or of panels of their rows.
 cudaError_t launch_slice_scales(SlMat* mats, int nmat, const SlProblem* probs, int nprob, void* ws, cudaStream_t s);
 // Up to 8 operands and 4 problems per call (K <= 65536); err as for launch_gemm_tc. ws holds the
 // operands' slices and the problems' lists.
-cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob,
+cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob, SliceBound bound,
                                bool accumulate, void* ws, size_t ws_bytes, int* err, cudaStream_t s);
 
 // A[p,u,l,d,r] (real) -> a~ blocks in FSO [(u,l)|(d,r)]; hermitian selects the

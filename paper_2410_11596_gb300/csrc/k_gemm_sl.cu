@@ -46,12 +46,14 @@
 // one MMA a K step), and an entry whose error bound
 //   2^-56 2^(ea + eb) (sum |a| / 2^ea + sum |b| / 2^eb)      (operands' rounding)
 //   + the truncation of levels 7..9
-// exceeds 2 sqrt(K) 2^-53 S is listed, and fma_kernel sums it by FP64 FMAs. (A chain's
+// exceeds 2 sqrt(K) 2^-53 S (kBoundEntry) is listed, and fma_kernel sums it by FP64 FMAs. (A chain's
 // own worst case is K 2^-53 S, its error on random terms 0.5 2^-53 S, the slices' at the
 // bound 1 to 2 2^-53 S; operands whose halves of the index hold rows in turn, 100 times
 // larger: 0.59 as a chain, 3.2 with a bound of 4 sqrt(K), 0.59 with this one.) Entries of rows or columns that hold an infinity or NaN, or whose
 // scale leaves [2^-400, 2^500], are listed too, so non-finite values propagate as in a
-// chain. Root mean square of error / S in units of 2^-53, 10368 x 666 x 666, A falling
+// chain. The chains of the library, whose operands carry errors of 2^-53 of their
+// largest entries already, hold theirs to K 2^-53 S or to the rows' scale (SliceBound, where
+// it is chosen). Root mean square of error / S in units of 2^-53, 10368 x 666 x 666, A falling
 // and B rising by d decades along k; without scales and lists, with them, library DGEMM:
 //   d = 0: 0.05, 0.05, 0.47   2: 3.6, 0.10, 0.48   4: 285, 0.12, 0.49   8: 2e6, 0.10, 0.47
 // in 276 us before, 290 now. Of the CTMRG and HOTRG chains' entries some 1e-3 are listed
@@ -1217,7 +1219,8 @@ cudaError_t launch_slice_scales(SlMat* mats, int nmat, const SlProblem* probs, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob, bool accumulate,
+cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* probs, int nprob, SliceBound bound,
+                               bool accumulate,
                                void* ws, size_t ws_bytes, int* err, cudaStream_t s) {
   if (nmat > kMaxSplit || nprob > kMaxProblems || nprob < 1) return cudaErrorInvalidValue;
   SplitOp all[kMaxSplit] = {};
@@ -1269,15 +1272,20 @@ cudaError_t launch_gemm_slices(const SlMat* mats, int nmat, const SlProblem* pro
     u.eb = b.exps;
     u.ra = a.row;
     u.rb = b.row;
-    // bound <= b(K) 2^-53 S with b = 2 sqrt(K), and K - 1 where that is less. The 19
+    // bound <= b(K) 2^-53 S with b = 2 sqrt(K), and K - 1 (the last rounding takes one)
+    // where that is less or a chain's bound will do. The 19
     // pairs of levels 7..9 take one FP32 add (truncated) each per 16 columns, up to 192
     // columns; random digits sum to `low`, 8 times that means that they are not
-    const double sq = 2.0 * std::sqrt((double)u.K), bk = sq < u.K - 1.0 ? sq : u.K > 1 ? u.K - 1.0 : 1e-9;
+    const double sq = 2.0 * std::sqrt((double)u.K), bk = bound == kBoundEntry && sq < u.K - 1.0 ? sq : u.K > 1 ? u.K - 1.0 : 1e-9;
     const double adds = 19.0 * (u.K < CHUNK * KC ? (u.K + 15) / 16 : CHUNK * KC / 16);
     const double low = std::ldexp(std::sqrt(6.0 * u.K) / 3.0, 14 - 40);
     u.g_round = (float)(std::ldexp(1.0, 30 - 56 + 53) / bk);
     u.g_low = (float)(std::ldexp(adds * low, 30 - 14 - 23 + 53) / bk);
     u.low_max = (float)(8.0 * low);
+    if (bound == kBoundRows) {  // marked rows only
+      u.g_round = u.g_low = 0.f;
+      u.low_max = INFINITY;
+    }
     u.a = a.m;
     u.b = b.m;
     // |sum| < 1.01 2^46 K: the fraction takes the bits that are left of 62
