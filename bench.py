@@ -44,8 +44,8 @@ FLUSH_BYTES = 512 << 20
 # DRAM traffic per launch of the roofline kernel from one ncu capture, valid only
 # while the kernel source is unchanged (sha256 of the file, first 16 hex digits).
 NCU_TRAFFIC = {
-    # FP64 block GEMM by digit slices, one ncu capture of a 10368 x 666 x 666 product: its operand split and GEMM
-    "gemm_sl": {"bytes_per_launch": 239.4e6, "source_sha": "a70f7fc166e94f07"},
+    # FP64 block GEMM by digit slices, one ncu capture of a 10368 x 666 x 666 product: its five launches
+    "gemm_sl": {"bytes_per_launch": 256.0e6, "source_sha": "f8fafbed06fa2573"},
     # tensor-core GEMM, one ncu capture of two steady-state D=6 chi=144 moves: mean over its launches
     "gemm_tc_tf32x3": {"bytes_per_launch": 56.5e6, "source_sha": "751d5096e63fff00"},
     # the same capture, mean over its split-output launches (G2-G5, the dominant kernel)
@@ -643,7 +643,8 @@ def run_ours(args):
         src, key = "paper_2410_11596_gb300/csrc/k_gemm_sl.cu", "gemm_sl"
         bf16, how = measured_bf16_tflops()
         peak, bound = bf16 / 34, "tensor"
-        kname = "gemm_sl_kernel and its operand splits (Z2 block GEMM, 34 BF16 products of 8-bit digit slices)"
+        kname = ("gemm_sl_kernel with its operands' splits and scales and its entries' bounds (Z2 block GEMM, 34 BF16 "
+                 "products of 8-bit digit slices)")
         psrc = f"bf16 burst {bf16:.1f} TF/s (of {how}) / 34 digit products per FP64 product"
     else:
         # the dominant kernel: the split-output instantiation of the tcgen05 GEMM (the enlarged corner

@@ -424,7 +424,8 @@ hs_status hs_hotrg_init(hs_ctx ctx, const hs_z2_tensor* a, hs_z2_tensor* t, doub
  * left); one FP64 eigen-decomposition per parity block, states kept across
  * both blocks by eigenvalue. A side one of whose decompositions fails is not
  * taken; HS_ERR_SOLVER if both fail. The new tensor is divided by its largest
- * modulus. precision: HS_PREC_F64 runs the block GEMMs on the FP64 kernel;
+ * modulus. precision: HS_PREC_F64 runs the block GEMMs in FP64 (as hs_gemm, but
+ * for an entry's error, which is held to its row's and column's scale);
  * HS_PREC_TF32X3 / TF32 / BF16X3 run them on tcgen05 (operands split straight
  * from their source layouts, FP32 accumulation, FP64 output); the Gram
  * eigen-decompositions are FP64 in every precision. info (host, may be NULL)
